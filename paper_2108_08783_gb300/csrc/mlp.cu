@@ -2,7 +2,9 @@
 // loss, back-propagation and Adam step, and the per-site feature / field
 // kernels that connect it to a lattice.  No counterpart in the paper.
 //
-// Every contraction (forward z = h W^T, input error d W, weight gradient
+// Networks up to 256 wide run in the whole-network kernels of
+// mlp_fused.cuh.  Wider ones (and one-layer ones) go layer by layer: every
+// contraction (forward z = h W^T, input error d W, weight gradient
 // d^T h) runs through one GEMM kernel on the fifth-generation tensor cores:
 // bfloat16 operands staged in shared memory in the canonical K-major layout,
 // tcgen05.mma (kind::f16, 128 x 128 x 16) accumulating in FP32 in tensor
@@ -358,6 +360,8 @@ __global__ void k_adam(float* th, const float* g, float* m, float* v, bf16* w16,
   }
 }
 
+#include "mlp_fused.cuh"
+
 int grid_for(int64_t n, int threads) {
   const int64_t b = (n + threads - 1) / threads;
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
@@ -443,6 +447,19 @@ struct lbm_mlp {
   bf16* d[2] = {nullptr, nullptr};  // errors, [max_batch][max(width, n_out)]
   double* loss = nullptr;
   int* dflag = nullptr;    // device flag: a bounded tensor-core wait gave up
+  // whole-network kernels (mlp_fused.cuh): the forward pass, and training
+  bool fused = false, fused_train = false;
+  FusedNet fnet{};
+  int n_sms = 1;
+  unsigned char* wpack = nullptr;  // weights as core-matrix images
+  int32_t* pmap = nullptr;         // byte offset of each weight in wpack, -1: bias
+  int32_t w_bytes = 0;             // weight buffer of k_mlp_train
+  int nb_max = 0;                  // its largest tile
+  int max_splits = 1;
+  unsigned char* img_h[kFusedLayers] = {};  // operand images of a training step
+  unsigned char* img_d[kFusedLayers] = {};
+  float* part = nullptr;           // [max_splits][n_params] partial gradients
+  double* loss_part = nullptr;     // [tiles][4]
   int64_t t = 0;           // Adam steps taken
   std::string err;
 };
@@ -472,6 +489,128 @@ void* malloc_dev(lbm_mlp* net, size_t bytes) {
   }
   if (p) net->owned.push_back(p);
   return p;
+}
+
+// ---------------------------------------------------- whole-network launches
+
+int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Rows per tile so that n rows fill whole rounds of `slots` tiles evenly, a
+// multiple of 16 up to `most` (65,536 rows on 2 x 152 slots: two rounds of
+// 112 rows, where 128 would leave the second round two thirds full).
+int tile_rows(int64_t n, int64_t slots, int most) {
+  const int64_t rounds = ceil_div(n, slots * most);
+  const int64_t rows = ceil_div(n, slots * rounds);
+  return (int)std::min<int64_t>(most, std::max<int64_t>(16, (rows + 15) / 16 * 16));
+}
+
+size_t train_smem(const lbm_mlp* net, int nb) {
+  return 128 + (size_t)net->w_bytes +
+         (size_t)nb * 16 * (4 + (size_t)(net->n_layers - 1) * net->fnet.l[0].rg);
+}
+
+// The layers' images and what the whole-network kernels can take: hidden
+// layers of at most 256, and for training all activations of a 16-row tile
+// beside the largest weight image in one SM's shared memory.
+void fused_plan(lbm_mlp* net) {
+  if (net->n_layers < 2 || net->n_layers > kFusedLayers || net->width > kFusedWidth) return;
+  FusedNet& f = net->fnet;
+  f.n_layers = net->n_layers;
+  f.n_in = net->n_in;
+  f.n_out = net->n_out;
+  uint32_t o = 0, wb = 0;
+  for (int l = 0; l < net->n_layers; ++l) {
+    FusedLayer& L = f.l[l];
+    L.rows = net->rows[l];
+    L.cols = net->cols[l];
+    L.rg = pad16(L.rows) / 8;
+    L.cg = pad16(L.cols) / 8;
+    L.pack = o;
+    L.w_off = (uint32_t)net->w_off[l];
+    L.b_off = (uint32_t)net->b_off[l];
+    o += (uint32_t)(L.rg * L.cg) * kCoreBytes;
+    // what a product may read: whole 128-row blocks forward, whole
+    // 128-column blocks of the last row group on the way back
+    const uint32_t fwd = (uint32_t)((L.rg + 15) / 16 * 16 * L.cg) * kCoreBytes;
+    const uint32_t back = (uint32_t)(L.rg * L.cg + 16) * kCoreBytes;
+    wb = std::max(wb, std::max(fwd, back));
+  }
+  net->fused = true;
+  net->w_bytes = (int32_t)wb;
+  int dev = 0, sms = 0, smem = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+    cudaGetLastError();
+    net->fused = false;
+    return;
+  }
+  net->n_sms = sms;
+  const int blocks = (net->width + 127) / 128;
+  net->max_splits = std::max(1, sms / (net->n_layers * blocks));
+  const size_t room = (size_t)smem - 1024;  // the kernel's barriers are static
+  for (int nb = kTrainRows; nb >= 16 && !net->nb_max; nb -= 16)
+    if (train_smem(net, nb) <= room) net->nb_max = nb;
+  net->fused_train = net->nb_max > 0;
+  bool ok = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kFwdSmem) == cudaSuccess &&
+            cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)room) == cudaSuccess &&
+            cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kGradRing + 128) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    net->fused = net->fused_train = false;
+  }
+}
+
+int fused_forward(lbm_mlp* net, const float* x, int64_t n, float* y, cudaStream_t s) {
+  if (n <= 0) return 0;
+  const int64_t slots = 2 * (int64_t)net->n_sms;
+  const int nb = tile_rows(n, slots, kFwdRows);
+  const int64_t tiles = ceil_div(n, nb);
+  k_mlp_forward<<<(unsigned)std::min(tiles, slots), kFwdThreads, kFwdSmem, s>>>(net->fnet, x, n,
+                                                                                nb, y);
+  return (int)cudaGetLastError();
+}
+
+// Loss parts and partial gradients of the batch; splits and loss parts used.
+int fused_grads(lbm_mlp* net, const float* x, const float* t, int64_t n, cudaStream_t s,
+                int* splits, int64_t* n_loss) {
+  const int64_t count = n * net->n_out;
+  TrainArgs a{};
+  a.net = net->fnet;
+  a.x = x;
+  a.t = t;
+  a.n = n;
+  a.nb = tile_rows(n, net->n_sms, net->nb_max);
+  a.w_bytes = net->w_bytes;
+  a.scale = (float)(2.0 / (double)count);
+  a.inv_count = 1.0 / (double)count;
+  a.loss_part = net->loss_part;
+  GradArgs g{};
+  g.net = net->fnet;
+  for (int l = 0; l < net->n_layers; ++l) {
+    g.h[l] = a.h[l] = net->img_h[l];
+    g.d[l] = a.d[l] = net->img_d[l];
+  }
+  const int64_t tiles = ceil_div(n, a.nb);
+  k_mlp_train<<<(unsigned)std::min<int64_t>(tiles, net->n_sms), kTrainThreads,
+                train_smem(net, a.nb), s>>>(a);
+  int e = (int)cudaGetLastError();
+  if (e) return e;
+  g.tiles = tiles;
+  g.nb = a.nb;
+  g.blocks = (net->width + 127) / 128;
+  g.splits = (int)std::min<int64_t>(tiles, net->max_splits);
+  g.stages = std::min(kGradMaxStages, kGradRing / (48 * 16 * a.nb));
+  g.part = net->part;
+  g.n_params = net->n_params;
+  k_mlp_wgrad<<<dim3((unsigned)(net->n_layers * g.blocks), (unsigned)g.splits), kGradThreads,
+                g.stages * 48 * 16 * a.nb + 128, s>>>(g);
+  *splits = g.splits;
+  *n_loss = 4 * tiles;
+  return (int)cudaGetLastError();
 }
 
 // Layer l reads h_l: the bfloat16 inputs (l = 0) or the activations h[l-1].
@@ -584,6 +723,7 @@ namespace lbm {
 
 int mlp_forward_on(lbm_mlp* net, const float* x, int64_t n, float* y, void* stream) {
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (net->fused) return fused_forward(net, x, n, y, s);  // no buffers: any number of rows
   for (int64_t r = 0; r < n; r += net->max_batch) {
     const int64_t m = std::min(net->max_batch, n - r);
     const int e = forward_rows(net, x + r * net->n_in, m, y + r * net->n_out, s);
@@ -668,12 +808,44 @@ int lbm_mlp_create(int32_t n_in, int32_t width, int32_t n_layers, int32_t n_out,
   net->m = f32(o);
   net->v = f32(o);
   net->w16 = b16(o);
-  net->x16 = b16(max_batch * n_in);
-  for (int l = 0; l + 1 < n_layers; ++l) net->h.push_back(b16(max_batch * width));
-  net->y = f32(max_batch * n_out);
-  const int dw = std::max(width, n_out);
-  net->d[0] = b16(max_batch * dw);
-  net->d[1] = b16(max_batch * dw);
+  fused_plan(net);
+  auto bytes = [&](int64_t count) {
+    unsigned char* p = static_cast<unsigned char*>(malloc_dev(net, count));
+    ok = ok && p;
+    return p;
+  };
+  std::vector<int32_t> pmap;
+  int64_t pack_bytes = 0;
+  if (net->fused) {
+    pmap.assign((size_t)o, -1);
+    for (int l = 0; l < n_layers; ++l) {
+      const FusedLayer& L = net->fnet.l[l];
+      pack_bytes = L.pack + (int64_t)L.rg * L.cg * kCoreBytes;
+      for (int r = 0; r < L.rows; ++r)
+        for (int c = 0; c < L.cols; ++c)
+          pmap[(size_t)L.w_off + (size_t)r * L.cols + c] =
+              (int32_t)(L.pack + ((r >> 3) * L.cg + (c >> 3)) * kCoreBytes + (r & 7) * 16 +
+                        (c & 7) * 2);
+    }
+    net->wpack = bytes(pack_bytes);
+    net->pmap = reinterpret_cast<int32_t*>(bytes(o * (int64_t)sizeof(int32_t)));
+  }
+  if (net->fused_train) {
+    const int64_t rows = max_batch + kTrainRows;  // whole tiles of any batch
+    for (int l = 0; l < n_layers; ++l) {
+      net->img_h[l] = bytes(rows * 16 * net->fnet.l[l].cg);
+      net->img_d[l] = bytes(rows * 16 * net->fnet.l[l].rg);
+    }
+    net->part = f32(net->max_splits * o);
+    net->loss_part = reinterpret_cast<double*>(bytes(4 * (rows / 16) * (int64_t)sizeof(double)));
+  } else {
+    net->x16 = b16(max_batch * n_in);
+    for (int l = 0; l + 1 < n_layers; ++l) net->h.push_back(b16(max_batch * width));
+    net->y = f32(max_batch * n_out);
+    const int dw = std::max(width, n_out);
+    net->d[0] = b16(max_batch * dw);
+    net->d[1] = b16(max_batch * dw);
+  }
   net->loss = static_cast<double*>(malloc_dev(net, sizeof(double)));
   net->dflag = static_cast<int*>(malloc_dev(net, sizeof(int)));
   ok = ok && net->loss && net->dflag;
@@ -687,6 +859,15 @@ int lbm_mlp_create(int32_t n_in, int32_t width, int32_t n_layers, int32_t n_out,
     if (!e) e = (int)cudaMemsetAsync(p, 0, o * sizeof(float), s);
   if (!e) e = (int)cudaMemsetAsync(net->w16, 0, o * sizeof(bf16), s);
   if (!e) e = (int)cudaMemsetAsync(net->dflag, 0, sizeof(int), s);
+  if (net->fused) {
+    net->fnet.wpack = net->wpack;
+    net->fnet.theta = net->theta;
+    net->fnet.err = net->dflag;
+    if (!e) e = (int)cudaMemsetAsync(net->wpack, 0, pack_bytes, s);  // the padding stays zero
+    if (!e)
+      e = (int)cudaMemcpyAsync(net->pmap, pmap.data(), pmap.size() * sizeof(int32_t),
+                               cudaMemcpyHostToDevice, s);
+  }
   if (!e) e = (int)cudaStreamSynchronize(s);
   if (e) {
     lbm_mlp_destroy(net);
@@ -715,6 +896,11 @@ int lbm_mlp_set_params(lbm_mlp* net, const float* theta, int32_t src_is_device) 
     k_to_bf16<<<grid_for(net->n_params, 256), 256, 0, s>>>(net->theta, net->w16, net->n_params);
     e = (int)cudaGetLastError();
   }
+  if (!e && net->fused) {
+    k_pack<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(net->w16, net->pmap, net->wpack,
+                                                                  net->n_params);
+    e = (int)cudaGetLastError();
+  }
   if (!e) e = (int)cudaStreamSynchronize(s);
   net->t = 0;
   return mcuda(net, e, "lbm_mlp_set_params");
@@ -741,7 +927,19 @@ int lbm_mlp_loss_grad(lbm_mlp* net, const float* x, const float* t, int64_t n, d
   if (!x || !t || !loss || n < 1 || n > net->max_batch)
     return mfail(net, LBM_EINVAL, "lbm_mlp_loss_grad: arguments");
   cudaStream_t s = net->stream;
-  int e = loss_grad_rows(net, x, t, n, s);
+  int e = 0;
+  if (net->fused_train) {
+    int splits = 0;
+    int64_t n_loss = 0;
+    e = fused_grads(net, x, t, n, s, &splits, &n_loss);
+    if (!e) {
+      k_grad_sum<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(
+          net->part, splits, net->n_params, net->loss_part, n_loss, net->grad, net->loss);
+      e = (int)cudaGetLastError();
+    }
+  } else {
+    e = loss_grad_rows(net, x, t, n, s);
+  }
   if (!e && grad)
     e = (int)cudaMemcpyAsync(grad, net->grad, net->n_params * sizeof(float),
                              (cudaMemcpyKind)copy_kind(dst_is_device, false), s);
@@ -758,15 +956,31 @@ int lbm_mlp_train_step(lbm_mlp* net, const float* x, const float* t, int64_t n,
       !(opt->eps > 0.0))
     return mfail(net, LBM_EINVAL, "lbm_mlp_train_step: arguments");
   cudaStream_t s = net->stream;
-  int e = loss_grad_rows(net, x, t, n, s);
+  int splits = 0;
+  int64_t n_loss = 0;
+  int e = net->fused_train ? fused_grads(net, x, t, n, s, &splits, &n_loss)
+                           : loss_grad_rows(net, x, t, n, s);
   if (e) return mcuda(net, e, "lbm_mlp_train_step");
   net->t += 1;
   const double c1 = 1.0 / (1.0 - std::pow(opt->beta1, (double)net->t));
   const double c2 = 1.0 / (1.0 - std::pow(opt->beta2, (double)net->t));
-  k_adam<<<grid_for(net->n_params, 256), 256, 0, s>>>(
-      net->theta, net->grad, net->m, net->v, net->w16, net->n_params, (float)opt->lr,
-      (float)opt->beta1, (float)opt->beta2, (float)opt->eps, (float)c1, (float)c2);
-  e = (int)cudaGetLastError();
+  if (net->fused_train) {
+    k_adam_fused<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(
+        net->theta, net->part, splits, net->m, net->v, net->w16, net->pmap, net->wpack,
+        net->n_params, (float)opt->lr, (float)opt->beta1, (float)opt->beta2, (float)opt->eps,
+        (float)c1, (float)c2, net->loss_part, n_loss, net->loss);
+    e = (int)cudaGetLastError();
+  } else {
+    k_adam<<<grid_for(net->n_params, 256), 256, 0, s>>>(
+        net->theta, net->grad, net->m, net->v, net->w16, net->n_params, (float)opt->lr,
+        (float)opt->beta1, (float)opt->beta2, (float)opt->eps, (float)c1, (float)c2);
+    e = (int)cudaGetLastError();
+    if (!e && net->fused) {  // too deep for k_mlp_train: the forward pass still needs the images
+      k_pack<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(net->w16, net->pmap,
+                                                                    net->wpack, net->n_params);
+      e = (int)cudaGetLastError();
+    }
+  }
   if (!e && loss) {
     e = (int)cudaMemcpyAsync(loss, net->loss, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (!e) e = (int)cudaStreamSynchronize(s);
