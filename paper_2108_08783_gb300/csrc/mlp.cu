@@ -458,7 +458,7 @@ struct lbm_mlp {
   int max_splits = 1;
   unsigned char* img_h[kFusedLayers] = {};  // operand images of a training step
   unsigned char* img_d[kFusedLayers] = {};
-  float* part = nullptr;           // [max_splits][n_params] partial gradients
+  float* part = nullptr;           // [max_splits][part_stride] partial gradients
   double* loss_part = nullptr;     // [tiles][4]
   int64_t t = 0;           // Adam steps taken
   std::string err;
@@ -495,6 +495,9 @@ void* malloc_dev(lbm_mlp* net, size_t bytes) {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Row length of the partial gradients.
+int64_t part_stride(const lbm_mlp* net) { return (net->n_params + 3) / 4 * 4; }
+
 // Rows per tile so that n rows fill whole rounds of `slots` tiles evenly, a
 // multiple of 16 up to `most` (65,536 rows on 2 x 152 slots: two rounds of
 // 112 rows, where 128 would leave the second round two thirds full).
@@ -529,10 +532,10 @@ void fused_plan(lbm_mlp* net) {
     L.w_off = (uint32_t)net->w_off[l];
     L.b_off = (uint32_t)net->b_off[l];
     o += (uint32_t)(L.rg * L.cg) * kCoreBytes;
-    // what a product may read: whole 128-row blocks forward, whole
-    // 128-column blocks of the last row group on the way back
-    const uint32_t fwd = (uint32_t)((L.rg + 15) / 16 * 16 * L.cg) * kCoreBytes;
-    const uint32_t back = (uint32_t)(L.rg * L.cg + 16) * kCoreBytes;
+    // what a product may read: whole 128-row blocks of the last column group
+    // forward, whole 128-column blocks on the way back
+    const uint32_t fwd = (uint32_t)(L.rg * L.cg + 16) * kCoreBytes;
+    const uint32_t back = (uint32_t)((L.cg + 15) / 16 * 16 * L.rg) * kCoreBytes;
     wb = std::max(wb, std::max(fwd, back));
   }
   net->fused = true;
@@ -605,7 +608,7 @@ int fused_grads(lbm_mlp* net, const float* x, const float* t, int64_t n, cudaStr
   g.splits = (int)std::min<int64_t>(tiles, net->max_splits);
   g.stages = std::min(kGradMaxStages, kGradRing / (48 * 16 * a.nb));
   g.part = net->part;
-  g.n_params = net->n_params;
+  g.part_stride = part_stride(net);
   k_mlp_wgrad<<<dim3((unsigned)(net->n_layers * g.blocks), (unsigned)g.splits), kGradThreads,
                 g.stages * 48 * 16 * a.nb + 128, s>>>(g);
   *splits = g.splits;
@@ -824,7 +827,7 @@ int lbm_mlp_create(int32_t n_in, int32_t width, int32_t n_layers, int32_t n_out,
       for (int r = 0; r < L.rows; ++r)
         for (int c = 0; c < L.cols; ++c)
           pmap[(size_t)L.w_off + (size_t)r * L.cols + c] =
-              (int32_t)(L.pack + ((r >> 3) * L.cg + (c >> 3)) * kCoreBytes + (r & 7) * 16 +
+              (int32_t)(L.pack + ((c >> 3) * L.rg + (r >> 3)) * kCoreBytes + (r & 7) * 16 +
                         (c & 7) * 2);
     }
     net->wpack = bytes(pack_bytes);
@@ -836,7 +839,7 @@ int lbm_mlp_create(int32_t n_in, int32_t width, int32_t n_layers, int32_t n_out,
       net->img_h[l] = bytes(rows * 16 * net->fnet.l[l].cg);
       net->img_d[l] = bytes(rows * 16 * net->fnet.l[l].rg);
     }
-    net->part = f32(net->max_splits * o);
+    net->part = f32(net->max_splits * part_stride(net));
     net->loss_part = reinterpret_cast<double*>(bytes(4 * (rows / 16) * (int64_t)sizeof(double)));
   } else {
     net->x16 = b16(max_batch * n_in);
@@ -934,7 +937,7 @@ int lbm_mlp_loss_grad(lbm_mlp* net, const float* x, const float* t, int64_t n, d
     e = fused_grads(net, x, t, n, s, &splits, &n_loss);
     if (!e) {
       k_grad_sum<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(
-          net->part, splits, net->n_params, net->loss_part, n_loss, net->grad, net->loss);
+          net->part, splits, part_stride(net), net->n_params, net->loss_part, n_loss, net->grad, net->loss);
       e = (int)cudaGetLastError();
     }
   } else {
@@ -966,7 +969,7 @@ int lbm_mlp_train_step(lbm_mlp* net, const float* x, const float* t, int64_t n,
   const double c2 = 1.0 / (1.0 - std::pow(opt->beta2, (double)net->t));
   if (net->fused_train) {
     k_adam_fused<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(
-        net->theta, net->part, splits, net->m, net->v, net->w16, net->pmap, net->wpack,
+        net->theta, net->part, splits, part_stride(net), net->m, net->v, net->w16, net->pmap, net->wpack,
         net->n_params, (float)opt->lr, (float)opt->beta1, (float)opt->beta2, (float)opt->eps,
         (float)c1, (float)c2, net->loss_part, n_loss, net->loss);
     e = (int)cudaGetLastError();

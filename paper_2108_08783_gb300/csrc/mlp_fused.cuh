@@ -10,9 +10,10 @@
 // Every operand image is made of 8 x 8 core matrices of 128 contiguous bytes
 // (no swizzle), and each image serves two contractions by the descriptor's
 // transpose bits and strides alone:
-//   weights W_l, core (rg, cg) holding 8 rows (out features) of 8 columns (in
-//     features): K-major A of the forward product (M = rows, K = columns) and
-//     MN-major A of the input error (M = columns, K = rows);
+//   weights W_l, core (cg, rg) holding 8 rows (out features) of 8 columns (in
+//     features), column groups outermost: K-major A of the forward product
+//     (M = rows, K = columns) and MN-major A of the input error (M = columns,
+//     K = rows); any run of columns is one contiguous block;
 //   activations h_l and errors delta_l, core (fg, ng) holding 8 features of 8
 //     batch rows: MN-major B of the products above (N = rows, K = features)
 //     and K-major A or B of the weight gradient (K = batch rows).
@@ -172,17 +173,19 @@ __device__ __forceinline__ void stage_inputs(unsigned char* image, const float* 
 // y = network(x) for n rows.  A CTA takes tiles of nb <= 128 rows through all
 // layers: the activations stay in shared memory (64 KB, overwritten in place
 // once a layer's MMAs have read them), the packed weights stream from L2
-// through a ring of 16 KB stages (32 input features of the layer's rows each).
+// through a ring of 16 KB stages (32 input features of the layer's rows each, one
+// bulk copy: 32 copies of 512 bytes a stage held the products back to half rate).
 // Warps 0-7 are the epilogue, warp 8 fills the ring, one lane of warp 9 issues
 // the MMAs.  The epilogue's tanhf bounds it (50 M of them for 65,536 rows of
 // the 4 x 256 network), so two CTAs share an SM (2 x 112 KB of shared memory,
 // 2 x 256 accumulator columns): one's products run under the other's
 // epilogue.  nb is chosen so that the tiles fill whole rounds of 2 CTAs per SM.
-// 65,536 rows of the 4 x 256 network: 219 us layer by layer, 74 us so; a warm
-// start of 926,000 sites (226 chunks of 4,096 rows before): 21.1 -> 1.14 ms.
+// 65,536 rows of the 4 x 256 network: 219 us layer by layer, 59 us so; the
+// pass of a warm start of 926,000 sites (227 chunks of 4,096 rows before, about
+// 20 ms): 0.72 ms, at 2.4 warp instructions a cycle and SM.
 constexpr int kFwdStages = 3;
 constexpr int kStageBytes = 32 * 4 * kCoreBytes;  // 256 rows x 32 columns
-constexpr int kFwdEpiWarps = 8;
+constexpr int kFwdEpiWarps = 8;  // 8 or 16 (16 measured no faster)
 constexpr int kFwdThreads = (kFwdEpiWarps + 2) * 32;
 constexpr uint32_t kFwdTmem = 256;
 constexpr int kFwdSmem = 32 * (kFwdRows / 8) * kCoreBytes + kFwdStages * kStageBytes + 128;
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   unsigned char* ring = act + 32 * (kFwdRows / 8) * kCoreBytes;
   __shared__ __align__(8) FwdBars s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == 9) tc_alloc(&s.tmem, kFwdTmem);
+  if (warp == kFwdEpiWarps + 1) tc_alloc(&s.tmem, kFwdTmem);
   if (tid == 0) {
     for (int i = 0; i < kFwdStages; ++i) {
       mbar_init_n(&s.full[i], 1);
@@ -217,7 +220,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   const int64_t tiles = (n + nb - 1) / nb;
   const uint32_t kstr = (uint32_t)nb * 16;  // feature-group stride of the activations
 
-  if (warp == 8) {
+  if (warp == kFwdEpiWarps) {
     // ring producer: chunks of 4 column groups of every layer of every tile
     uint32_t it = 0;
     bool ok = true;
@@ -230,13 +233,12 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
             ok = false;
             break;
           }
-          const uint32_t part = (uint32_t)min(4, L.cg - c) * kCoreBytes;
-          if (lane == 0) mbar_expect(&s.full[st], part * (uint32_t)L.rg);
-          __syncwarp();
-          if (lane < L.rg)
-            copy_g2s(ring + st * kStageBytes + lane * 4 * kCoreBytes,
-                     net.wpack + L.pack + (uint32_t)(lane * L.cg + c) * kCoreBytes, part,
-                     &s.full[st]);
+          const uint32_t bytes = (uint32_t)(min(4, L.cg - c) * L.rg) * kCoreBytes;
+          if (lane == 0) {
+            mbar_expect(&s.full[st], bytes);
+            copy_g2s(ring + st * kStageBytes, net.wpack + L.pack + (uint32_t)(c * L.rg) * kCoreBytes,
+                     bytes, &s.full[st]);
+          }
         }
       }
     if (!ok) {
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
       // copies in flight get one more (bounded) chance to land
       for (int i = 0; i < kFwdStages; ++i) mbar_wait(&s.full[i], 0);
     }
-  } else if (warp == 9) {
+  } else if (warp == kFwdEpiWarps + 1) {
     if (lane == 0) {
       uint32_t it = 0, step = 0;
       bool ok = true;
@@ -253,6 +255,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
           const FusedLayer& L = net.l[l];
           const int mt = (L.rg + 15) / 16;
           const uint32_t idesc = mma_desc(nb, false, true);
+          const uint32_t rstr = (uint32_t)L.rg * kCoreBytes;  // column-group stride
           ok = mbar_wait(&s.ready, step & 1u);
           tc_after();
           for (int c = 0; c < L.cg && ok; c += 4, ++it) {
@@ -263,8 +266,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
             for (int m = 0; m < mt; ++m)
               for (int k = 0; k < 4 && c + k < L.cg; k += 2)
                 tc_mma(tmem + (uint32_t)(m * nb),
-                       core_desc(a0 + (uint32_t)(m * 16 * 4 + k) * kCoreBytes, kCoreBytes,
-                                 4 * kCoreBytes),
+                       core_desc(a0 + (uint32_t)(m * 16) * kCoreBytes + k * rstr, rstr, kCoreBytes),
                        core_desc(saddr(act) + (uint32_t)(c + k) * kstr, kstr, kCoreBytes), idesc,
                        c + k > 0);
             tc_commit(&s.empty[st]);
@@ -275,7 +277,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
     }
     __syncwarp();
   } else {
-    const int q = warp & 3, half = warp >> 2;
+    constexpr int kRowsets = kFwdEpiWarps / 4;  // warps of each 32-feature row set
+    const int q = warp & 3, set = warp >> 2;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     uint32_t step = 0;
     bool ok = true;
@@ -289,42 +292,42 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
       for (int l = 0; l < net.n_layers; ++l, ++step) {
         const FusedLayer& L = net.l[l];
         const bool last = l + 1 == net.n_layers;
-        // two accumulator tiles: a half of the warps each; one: half the columns each
+        // two accumulator tiles: half of the row sets each, and the 8-row column
+        // groups dealt out among the warps of a row set
         const bool two = L.rg > 16;
-        const int f = (two ? half * 128 : 0) + q * 32 + lane;
+        const int part = two ? set >> 1 : set, parts = two ? kRowsets / 2 : kRowsets;
+        const int f = (two ? (set & 1) * 128 : 0) + q * 32 + lane;
         const float bias = f < L.rows ? __ldg(net.theta + L.b_off + f) : 0.0f;
         if (!__all_sync(0xffffffffu, mbar_wait(&s.acc, step & 1u))) {
           ok = false;
           break;
         }
         tc_after();
-        const uint32_t base = lane_addr + (two ? (uint32_t)(half * nb) : 0u);
+        const uint32_t base = lane_addr + (two ? (uint32_t)((set & 1) * nb) : 0u);
         if (last) {
           if (q == 0)
-            for (int c0 = half * 16; c0 < nb; c0 += 32) {
-              float v[16];
-              tc_ld16(base + c0, v);
+            for (int c0 = part * 8; c0 < nb; c0 += parts * 8) {
+              float v[8];
+              tc_ld8(base + c0, v);
               if (lane < net.n_out) {
                 float* o = y + (row0 + c0) * net.n_out + lane;
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
+                for (int j = 0; j < 8; ++j)
                   if (c0 + j < valid) o[j * net.n_out] = v[j] + bias;
               }
             }
         } else {
           const bool keep = f < L.rg * 8;  // features the next layer reads
           unsigned char* row = act + (f >> 3) * kstr + (f & 7) * 16;
-          for (int c0 = two ? 0 : half * 16; c0 < nb; c0 += two ? 16 : 32) {
-            float v[16];
-            tc_ld16(base + c0, v);
+          for (int c0 = part * 8; c0 < nb; c0 += parts * 8) {
+            float v[8];
+            tc_ld8(base + c0, v);
             if (!keep) continue;
-            uint32_t w[8];
+            uint32_t w[4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
+            for (int j = 0; j < 4; ++j)
               w[j] = bf16_pair(tanhf(v[2 * j] + bias), tanhf(v[2 * j + 1] + bias));
-            uint4* o = reinterpret_cast<uint4*>(row + (c0 >> 3) * kCoreBytes);
-            o[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            o[kCoreBytes / 16] = make_uint4(w[4], w[5], w[6], w[7]);
+            *reinterpret_cast<uint4*>(row + (c0 >> 3) * kCoreBytes) = make_uint4(w[0], w[1], w[2], w[3]);
           }
           fence_async();
           tc_before();
@@ -336,7 +339,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   }
   tc_before();
   __syncthreads();
-  if (warp == 9) {
+  if (warp == kFwdEpiWarps + 1) {
     tc_after();
     tc_free(tmem, kFwdTmem);
   }
@@ -352,7 +355,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
 // batch of 4,096) spread the tanhf over all SMs: what bounds a step at the
 // study's batch is the chain of 2 n_layers - 1 dependent products.  A training
 // step of 4,096 rows of the 4 x 256 network, all kernels: 1,134 us layer by
-// layer, 61 us so.
+// layer, 45 us so (this kernel 22, the weight gradients 12, the optimiser 8).
 constexpr int kTrainEpiWarps = 16;
 constexpr int kTrainThreads = (kTrainEpiWarps + 2) * 32;
 constexpr uint32_t kTrainTmem = 128;
@@ -448,15 +451,15 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
           unsigned char* b = fwd ? image(l) : image(l + 1);
           const uint32_t bytes = (uint32_t)(fwd ? L.cg : L.rg) * kstr;
           const int mt = ((fwd ? L.rg : L.cg) + 15) / 16, ks = fwd ? L.cg : L.rg;
-          const uint32_t rstr = (uint32_t)L.cg * kCoreBytes;
+          const uint32_t rstr = (uint32_t)L.rg * kCoreBytes;  // column-group stride
           const uint32_t idesc = mma_desc(nb, !fwd, true);
           for (int m = 0; m < mt; ++m)
             for (int k = 0; k < ks; k += 2) {
               const uint64_t ad =
-                  fwd ? core_desc(saddr(wbuf) + (uint32_t)(m * 16) * rstr + k * kCoreBytes,
-                                  kCoreBytes, rstr)
-                      : core_desc(saddr(wbuf) + (uint32_t)(m * 16) * kCoreBytes + k * rstr, rstr,
-                                  kCoreBytes);
+                  fwd ? core_desc(saddr(wbuf) + (uint32_t)(m * 16) * kCoreBytes + k * rstr, rstr,
+                                  kCoreBytes)
+                      : core_desc(saddr(wbuf) + (uint32_t)(m * 16) * rstr + k * kCoreBytes,
+                                  kCoreBytes, rstr);
               tc_mma(tmem + (uint32_t)(m * nb), ad, core_desc(saddr(b) + k * kstr, kstr, kCoreBytes),
                      idesc, k > 0);
             }
@@ -613,8 +616,8 @@ struct GradArgs {
   int64_t tiles;
   int32_t nb, splits, blocks;  // blocks: 128-feature blocks per layer
   int32_t stages;
-  float* part;               // [splits][n_params]
-  int64_t n_params;
+  float* part;               // [splits][part_stride]
+  int64_t part_stride;       // n_params rounded up to 4: rows stay 16-byte aligned
 };
 
 struct GradBars {
@@ -656,7 +659,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_wgrad(const __grid_cons
   __syncthreads();
   tc_after();
   const uint32_t tmem = s.tmem;
-  float* part = a.part + blockIdx.y * a.n_params;
+  float* part = a.part + blockIdx.y * a.part_stride;
   bool ok = true;
   if (warp == kGradEpiWarps) {
     if (lane == 0) {
@@ -761,10 +764,10 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_wgrad(const __grid_cons
 }
 
 // Sum of a parameter's partial gradients, in the order of the splits.
-__device__ __forceinline__ float grad_of(const float* part, int splits, int64_t n, int64_t i) {
+__device__ __forceinline__ float grad_of(const float* part, int splits, int64_t stride, int64_t i) {
   float g = 0.0f;
 #pragma unroll 8
-  for (int k = 0; k < splits; ++k) g += __ldg(part + k * n + i);
+  for (int k = 0; k < splits; ++k) g += __ldg(part + k * stride + i);
   return g;
 }
 // The loss from its per-tile parts, in a fixed order, by one warp.
@@ -776,23 +779,23 @@ __device__ __forceinline__ void loss_of(const double* part, int64_t n, double* l
   if (threadIdx.x == 0) *loss = v;
 }
 
-__global__ void k_grad_sum(const float* part, int splits, int64_t n, const double* loss_part,
+__global__ void k_grad_sum(const float* part, int splits, int64_t stride, int64_t n, const double* loss_part,
                            int64_t n_loss, float* grad, double* loss) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) grad[i] = grad_of(part, splits, n, i);
+  if (i < n) grad[i] = grad_of(part, splits, stride, i);
   if (blockIdx.x == 0 && threadIdx.x < 32) loss_of(loss_part, n_loss, loss);
 }
 
 // k_adam on the summed partial gradients; also writes the packed weights
 // (pmap: byte offset of a weight in the images, -1 for a bias).
-__global__ void k_adam_fused(float* th, const float* part, int splits, float* m, float* v,
+__global__ void k_adam_fused(float* th, const float* part, int splits, int64_t stride, float* m, float* v,
                              bf16* w16, const int32_t* pmap, unsigned char* wpack, int64_t n,
                              float lr, float b1, float b2, float eps, float c1, float c2,
                              const double* loss_part, int64_t n_loss, double* loss) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.x == 0 && threadIdx.x < 32) loss_of(loss_part, n_loss, loss);
   if (i >= n) return;
-  const float gi = grad_of(part, splits, n, i);
+  const float gi = grad_of(part, splits, stride, i);
   const float mi = b1 * m[i] + (1.0f - b1) * gi;
   const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
   m[i] = mi;
