@@ -175,7 +175,21 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 __device__ __forceinline__ float recip(float v) { return __frcp_rn(v); }
-__device__ __forceinline__ double recip(double v) { return __drcp_rn(v); }
+
+// Estimates of 1/v that inv_one_plus below refines: to FP32 rounding, and for
+// FP64 to about 2^-40 (the hardware's 2^-20 and one Newton step). GB300's FP64
+// pipe takes one warp instruction per SM in 16 cycles, so a correctly rounded
+// reciprocal would be paid for twice.
+__device__ __forceinline__ float rcp_estimate(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ double rcp_estimate(double v) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  return __fma_rn(r, __fma_rn(-v, r, 1.0), r);
+}
 
 // Explicitly rounded multiply and fused multiply-add.  The boundary rule below
 // is written once and evaluated in an unrolled and a looped form; pinning its
@@ -295,23 +309,90 @@ __device__ __forceinline__ Mom<C> moments(const C (&g)[kQ]) {
   const C jy = (a3 + a7) - (a9 - a15) + a17;
   const C jz = (a5 + a11) - (a13 - a15) - a17;
   m.rho = C(1) + m.drho;
-  const C inv = inv_one_plus(m.drho, m.rho, recip(m.rho));
-  m.ux = jx * inv;
-  m.uy = jy * inv;
-  m.uz = jz * inv;
-  m.usq = C(1.5) * (m.ux * m.ux + m.uy * m.uy + m.uz * m.uz);
+  const C inv = inv_one_plus(m.drho, m.rho, rcp_estimate(m.rho));
+  m.ux = mul_pin(jx, inv);
+  m.uy = mul_pin(jy, inv);
+  m.uz = mul_pin(jz, inv);
+  m.usq = mul_pin(C(1.5), fma_pin(m.uz, m.uz, fma_pin(m.uy, m.uy, mul_pin(m.ux, m.ux))));
   return m;
 }
 
-// BGK relaxation (Eq. LBE_SRT): gs_i = g_i + omega (g^eq_i - g_i).
+// BGK relaxation (Eq. LBE_SRT), g*_i = g_i + omega (g^eq_i - g_i), pair by
+// opposite pair (a, b = a + 1): with cu = c_a.u = -c_b.u the equilibria are
+//   g^eq_a, g^eq_b = even +- l cu,  even = w (drho + rho (4.5 cu^2 - 1.5 u.u)),
+//   l = 3 w rho.
+// Two forms; in both every operation is written out (nothing is left to the
+// compiler to contract), so that all kernels round alike.
+//
+// Plain (FP32 storage, and every boundary tile): 9 operations a pair beyond cu,
+// where adding and subtracting the odd part took 10. The coefficients are one
+// rounding away from rho and drho, as rounding errors they share are not
+// averaged out over the directions: the scaled form below left the fields of
+// FP32 runs 1.3 to 1.5 times further from FP64.
+// Scaled (16-bit storage, whose rounding is 2^13 times coarser, and FP64, where
+// the operations are what a site costs): omega and the weights multiplied into
+//   omega g^eq = k + h cu^2 +- l cu,  k = omega w (drho - 1.5 rho u.u),
+//   h = 4.5 omega w rho,  l = 3 omega w rho,  g* = (1 - omega) g + omega g^eq:
+// 6 operations a pair.
+// The coefficients are those of the axis directions (w = 1/18); next() halves
+// them (exactly) for the diagonals. Every weight is a multiple of the FP32
+// 1/18 (7e-9 off): 1/6 for the odd part or 1/3 for the rest population, 3e-8
+// off, would change the momentum or the mass by the same fraction at every
+// step, and were the larger part of the error of FP32 runs (40 steps of the
+// long tube: 1.2e-6 to 1.7e-6 before, 0.6e-6 so).
+template <class C, bool SCALED>
+struct Relax;
 template <class C>
-__device__ __forceinline__ void relax(const C (&g)[kQ], C (&gs)[kQ], const Mom<C>& m, C omega) {
-  unroll<kQ>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    const C e = geq<i, C>(m.drho, m.rho, m.ux, m.uy, m.uz, m.usq);
-    gs[i] = g[i] + omega * (e - g[i]);
-  });
-}
+struct Relax<C, false> {
+  C omega, usq, wd, wr, l;
+  __device__ __forceinline__ Relax(const Mom<C>& m, C om)
+      : omega(om), usq(m.usq), wd(mul_pin(m.drho, C(1.0 / 18.0))),
+        wr(mul_pin(m.rho, C(1.0 / 18.0))), l(mul_pin(C(3), wr)) {}
+  __device__ __forceinline__ void next() {
+    wd *= C(0.5);
+    wr *= C(0.5);
+    l *= C(0.5);
+  }
+  __device__ __forceinline__ C rest(const Mom<C>& m, C g0) const {
+    const C e = mul_pin(C(6), mul_pin(C(1.0 / 18.0), fma_pin(-m.rho, m.usq, m.drho)));
+    return fma_pin(omega, e - g0, g0);
+  }
+  // also the parts a boundary needs: q = 4.5 cu^2 - 1.5 u.u, ea = g^eq_a - g_a, eb
+  __device__ __forceinline__ void pair(C cu, C ga, C gb, C& sa, C& sb, C& q, C& ea, C& eb) const {
+    q = fma_pin(mul_pin(C(4.5), cu), cu, -usq);
+    const C even = fma_pin(wr, q, wd);
+    ea = fma_pin(l, cu, even) - ga;
+    eb = fma_pin(-l, cu, even) - gb;
+    sa = fma_pin(omega, ea, ga);
+    sb = fma_pin(omega, eb, gb);
+  }
+  __device__ __forceinline__ void pair(C cu, C ga, C gb, C& sa, C& sb) const {
+    C q, ea, eb;
+    pair(cu, ga, gb, sa, sb, q, ea, eb);
+  }
+};
+template <class C>
+struct Relax<C, true> {
+  C keep, k, h, l, k0;
+  __device__ __forceinline__ Relax(const Mom<C>& m, C om) : keep(C(1) - om) {
+    const C kc = mul_pin(om, fma_pin(-m.rho, m.usq, m.drho)), wr = mul_pin(om, m.rho);
+    k = mul_pin(kc, C(1.0 / 18.0));
+    k0 = mul_pin(C(6), k);
+    h = mul_pin(wr, C(4.5 / 18.0));
+    l = mul_pin(C(3), mul_pin(wr, C(1.0 / 18.0)));
+  }
+  __device__ __forceinline__ void next() {
+    k *= C(0.5);
+    h *= C(0.5);
+    l *= C(0.5);
+  }
+  __device__ __forceinline__ C rest(const Mom<C>&, C g0) const { return fma_pin(keep, g0, k0); }
+  __device__ __forceinline__ void pair(C cu, C ga, C gb, C& sa, C& sb) const {
+    const C e = fma_pin(mul_pin(h, cu), cu, k);
+    sa = fma_pin(keep, ga, fma_pin(l, cu, e));
+    sb = fma_pin(keep, gb, fma_pin(-l, cu, e));
+  }
+};
 
 template <class C>
 __device__ __forceinline__ bool unstable(C rho) {
@@ -441,6 +522,16 @@ __device__ __forceinline__ bool chk_site(int64_t y, int64_t n, int* err) {
   return true;
 }
 
+// A copy of a base pointer the compiler cannot identify with the original:
+// stores through it form their addresses anew instead of keeping the 19 load
+// addresses live through the collision (38 registers on even steps).
+template <class S>
+__device__ __forceinline__ S* opaque_base(S* p) {
+  S* q;
+  asm volatile("mov.b64 %0, %1;" : "=l"(q) : "l"(p));
+  return q;
+}
+
 // Branch-free update of a site whose 18 links are fluid.
 // Returns the site's rho - 1 (for the fused mass diagnostic).  With SLOT the
 // whole warp (every lane updating a site) adds the lanes' rho - 1 as soon as
@@ -466,22 +557,15 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
     if ((threadIdx.x & 31) == 0) *slot = (double)sum;
   }
   if (unstable(m.rho)) atomicOr(err, kErrUnstable);
-  Cd::st(P + x, 0, g[0] + omega * (geq<0, C>(m.drho, m.rho, m.ux, m.uy, m.uz, m.usq) - g[0]));
+  Relax<C, !std::is_same<S, float>::value> rx(m, omega);
+  S* const Q = ODD ? P : opaque_base(P);
+  Cd::st(Q + x, 0, rx.rest(m, g[0]));
   chk_count(chk, P, P + x, kQ * np, err);
-  // Opposite directions a, b = opp(a) share c_b = -c_a, so their shifted
-  // equilibria split into an even part w (drho + rho (4.5 cu^2 - 1.5 u^2)) and
-  // an odd part 3 w rho cu: g^eq_a = even + odd, g^eq_b = even - odd.
-  const C wd1 = m.drho * C(1.0 / 18.0), wd2 = m.drho * C(1.0 / 36.0);
-  const C wr1 = m.rho * C(1.0 / 18.0), wr2 = m.rho * C(1.0 / 36.0);
-  const C w3r1 = m.rho * C(3.0 / 18.0), w3r2 = m.rho * C(3.0 / 36.0);
   unroll<9>([&](auto Pi) {
     constexpr int a = 2 * decltype(Pi)::value + 1, b = a + 1;
-    const C cu = cdot<a, C>(m.ux, m.uy, m.uz);
-    const C q = C(4.5) * cu * cu - m.usq;
-    const C even = (a <= 6) ? wd1 + wr1 * q : wd2 + wr2 * q;
-    const C odd = ((a <= 6) ? w3r1 : w3r2) * cu;
-    const C sa = g[a] + omega * ((even + odd) - g[a]);
-    const C sb = g[b] + omega * ((even - odd) - g[b]);
+    C sa, sb;
+    if constexpr (a == 7) rx.next();  // the first diagonal
+    rx.pair(cdot<a, C>(m.ux, m.uy, m.uz), g[a], g[b], sa, sb);
     if constexpr (ODD) {
       // The store to (x + c_a, a) hits the address the load of direction
       // opp(a) used; re-reading the offset from shared memory keeps the
@@ -493,8 +577,8 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
       chk_count(chk, P, pa, kQ * np, err);
       chk_count(chk, P, pb, kQ * np, err);
     } else {
-      Cd::st(P + b * np + x, a, sa);
-      Cd::st(P + a * np + x, b, sb);
+      Cd::st(Q + b * np + x, a, sa);
+      Cd::st(Q + a * np + x, b, sb);
       chk_count(chk, P, P + b * np + x, kQ * np, err);
       chk_count(chk, P, P + a * np + x, kQ * np, err);
     }
@@ -510,7 +594,7 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
 // (FP32) word, an odd offset as two scalars; the collision runs on packed
 // pairs with the two-wide FP32 instructions (add/sub/mul/fma .f32x2), so each
 // floating-point instruction serves both sites.  The arithmetic is that of
-// bulk_update, with the reciprocal of rho from the hardware approximation.
+// bulk_update.
 struct F2 {
   unsigned long long v;  // low word: site x, high word: site x + 1
 };
@@ -541,11 +625,6 @@ __device__ __forceinline__ F2 mul2(F2 a, F2 b) {
 __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {  // a b + c
   F2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ float rcp_approx(float v) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
   return r;
 }
 
@@ -649,7 +728,7 @@ __device__ __forceinline__ void chk_count2(int* chk, const S* P0, const S* p, in
 // for the relaxation (the 16-bit paths unpack them twice from packed words
 // rather than hold 38 floats); store0(g*_0) receives the rest population and
 // store<a, b>(g*_a, g*_b) those of each opposite pair (a odd, b = a + 1).
-template <class GetM, class GetP, class St0, class St>
+template <bool SCALED, class GetM, class GetP, class St0, class St>
 __device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, int* err_lo,
                                        int* err_hi, St0&& store0, St&& store) {
   // Eqs. (Density), (Momentum), grouped as in moments()
@@ -676,20 +755,30 @@ __device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, int* err_
   if (unstable(r1)) atomicOr(err_hi, kErrUnstable);
   float d0, d1;
   split2(drho, d0, d1);
-  const F2 inv = mk2(inv_one_plus(d0, r0, rcp_approx(r0)), inv_one_plus(d1, r1, rcp_approx(r1)));
+  const F2 inv = mk2(inv_one_plus(d0, r0, rcp_estimate(r0)), inv_one_plus(d1, r1, rcp_estimate(r1)));
   const F2 ux = mul2(jx, inv), uy = mul2(jy, inv), uz = mul2(jz, inv);
   const F2 usq = mul2(bc2(1.5f), fma2(uz, uz, fma2(uy, uy, mul2(ux, ux))));
-  // rest population: g*_0 = g_0 + omega (w_0 (drho - rho usq) - g_0)
-  const F2 e0 = mul2(bc2(1.0f / 3.0f), sub2(drho, mul2(rho, usq)));
-  {
+  // the two forms of Relax; m is -l, for the second direction of a pair
+  const F2 keep = sub2(bc2(1.0f), omega), nusq = sub2(bc2(0.0f), usq);
+  F2 k, h, l, m;  // plain: k = wd, h = wr
+  if constexpr (SCALED) {
+    const F2 kc = mul2(omega, fma2(rho, nusq, drho));
+    const F2 wr = mul2(omega, rho);
+    k = mul2(kc, bc2(1.0f / 18.0f));
+    store0(fma2(keep, gp(0), mul2(bc2(6.0f), k)));
+    h = mul2(wr, bc2(4.5f / 18.0f));
+    const F2 w18 = mul2(wr, bc2(1.0f / 18.0f));
+    l = mul2(bc2(3.0f), w18);
+    m = mul2(bc2(-3.0f), w18);
+  } else {
     const F2 g0 = gp(0);
+    const F2 e0 = mul2(bc2(6.0f), mul2(bc2(1.0f / 18.0f), fma2(rho, nusq, drho)));
     store0(fma2(omega, sub2(e0, g0), g0));
+    k = mul2(drho, bc2(1.0f / 18.0f));
+    h = mul2(rho, bc2(1.0f / 18.0f));
+    l = mul2(bc2(3.0f), h);
+    m = mul2(bc2(-3.0f), h);
   }
-  // opposite pairs (a, b): g^eq = even +- odd (see bulk_update)
-  const F2 wd1 = mul2(drho, bc2(1.0f / 18.0f)), wd2 = mul2(drho, bc2(1.0f / 36.0f));
-  const F2 wr1 = mul2(rho, bc2(1.0f / 18.0f)), wr2 = mul2(rho, bc2(1.0f / 36.0f));
-  const F2 w3r1 = mul2(rho, bc2(3.0f / 18.0f)), w3r2 = mul2(rho, bc2(3.0f / 36.0f));
-  const F2 nusq = sub2(bc2(0.0f), usq);
   unroll<9>([&](auto Pi) {
     constexpr int a = 2 * decltype(Pi)::value + 1;
     constexpr int pp = (a + 1) / 2;
@@ -703,12 +792,23 @@ __device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, int* err_
     else if constexpr (pp == 7) cu = sub2(ux, uz);
     else if constexpr (pp == 8) cu = add2(uy, uz);
     else cu = sub2(uy, uz);
-    const F2 q = fma2(mul2(bc2(4.5f), cu), cu, nusq);
-    const F2 even = (a <= 6) ? fma2(wr1, q, wd1) : fma2(wr2, q, wd2);
-    const F2 odd = mul2((a <= 6) ? w3r1 : w3r2, cu);
-    const F2 ga = gp(a), gb = gp(a + 1);
-    const F2 sa = fma2(omega, sub2(add2(even, odd), ga), ga);
-    const F2 sb = fma2(omega, sub2(sub2(even, odd), gb), gb);
+    if constexpr (a == 7) {  // the first diagonal: half the weight
+      k = mul2(k, bc2(0.5f));
+      h = mul2(h, bc2(0.5f));
+      l = mul2(l, bc2(0.5f));
+      m = mul2(m, bc2(0.5f));
+    }
+    F2 sa, sb;
+    if constexpr (SCALED) {
+      const F2 e = fma2(mul2(h, cu), cu, k);
+      sa = fma2(keep, gp(a), fma2(l, cu, e));
+      sb = fma2(keep, gp(a + 1), fma2(m, cu, e));
+    } else {
+      const F2 e = fma2(h, fma2(mul2(bc2(4.5f), cu), cu, nusq), k);
+      const F2 ga = gp(a), gb = gp(a + 1);
+      sa = fma2(omega, sub2(fma2(l, cu, e), ga), ga);
+      sb = fma2(omega, sub2(fma2(m, cu, e), gb), gb);
+    }
     store(std::integral_constant<int, a>{}, sa, sb);
   });
   return drho;
@@ -754,10 +854,11 @@ __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const
     if constexpr (kPacked) return Cd::unpack(opaque(r[j]));
     else return g[j];
   };
-  return sum2(collide2(
+  S* const Q = ODD ? P : opaque_base(P);
+  return sum2(collide2<sizeof(S) == 2>(
       gm, gp, bc2(omega), err, err,
       [&](F2 s0) {
-        Cd::st_al(P + x, s0);
+        Cd::st_al(Q + x, s0);
         chk_count2(chk, P, P + x, kQ * np, err);
       },
       [&](auto A, F2 sa, F2 sb) {
@@ -773,8 +874,8 @@ __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const
           chk_count2(chk, P, pa, kQ * np, err);
           chk_count2(chk, P, pb, kQ * np, err);
         } else {
-          Cd::st_al(P + b * np + x, sa);
-          Cd::st_al(P + a * np + x, sb);
+          Cd::st_al(Q + b * np + x, sa);
+          Cd::st_al(Q + a * np + x, sb);
           chk_count2(chk, P, P + b * np + x, kQ * np, err);
           chk_count2(chk, P, P + a * np + x, kQ * np, err);
         }
@@ -824,7 +925,7 @@ __device__ __forceinline__ float bulk_update2v(S* P, int64_t np, int64_t xa, int
     chk_count(chk, P, pa, kQ * np, err);
     chk_count(chk, P, pb, kQ * np, err);
   };
-  return sum2(collide2(
+  return sum2(collide2<sizeof(S) == 2>(
       gm, gp, bc2(omega), err, err,
       [&](F2 s0) { put(P + xa, SAME ? P + xa + kTile : P + xb, s0, 0); },
       [&](auto A, F2 sa, F2 sb) {
@@ -910,10 +1011,9 @@ constexpr int kAreaSite = 25;   // first row (compute-type units) of the per-sit
 //     state at an iolet link: (rho, u_in) at a velocity inlet, (rho_out, u) at a
 //     density outlet.  A fluid link i streams g*_i: into (x, j) on even steps,
 //     into (x + c_i, i) on odd steps.
-// warp_io / warp_wall (warp-uniform): some lane of the tile has iolet links /
-// elastic wall links, so their equilibria are computed at all; warp_nf: the
-// union of the tile's non-fluid directions (pairs no lane needs skip the
-// boundary values); site: the
+// wall_nf / io_nf (warp-uniform): the directions by which some lane of the tile
+// leaves the fluid through an elastic wall / an iolet (the equilibria of the
+// wall and iolet states are computed only for pairs that have one); site: the
 // warp's [5][32] per-site F, kappa/3, p0, ps, pc (copies in flight until
 // cp_async_wait_all); area: the warp's shared-memory area (BoundaryArea).
 // The odd-step slot deltas (opp(i) - i) np below stay within one row length
@@ -932,7 +1032,7 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
                                               const int32_t* offp, int ostride, uint32_t smask,
                                               uint32_t iom, const double* site,
                                               const int32_t* nbr_s, int lane, int64_t slot,
-                                              bool warp_io, bool warp_wall, uint32_t warp_nf,
+                                              uint32_t wall_nf, uint32_t io_nf,
                                               typename Codec<S>::C* area) {
   using Cd = Codec<S>;
   using C = typename Cd::C;
@@ -993,7 +1093,6 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
     else return g[j];
   };
   if (unstable(m.rho)) atomicOr(d.err, kErrUnstable);
-  const C keep = C(1) - omega;  // (1 - 1/tau)
   // Elastic wall (Sec. 2.3-2.4): dE in FP64, the ratio sw = U_w/u_f =
   // (F + dr - dx)/dr with dr = dx + dE in the compute type.
   C sw = C(0);
@@ -1018,12 +1117,11 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
       d.slot_Uw[2 * ss + slot] = (double)(sw * m.uz);
     }
   }
-  const C sw2 = sw * sw;
   // The site's iolet state (rho_b, u_b): velocity inlet (Sec. 3) u_in =
   // a (u_mean p0 + u_amp (ps sin th + pc cos th)) with rho_b = rho; density
   // outlet rho_b = rho_out with u_b = u.  Parked in the warp's shared-memory
   // area (read back only by tiles with iolet links), not held in registers.
-  if (warp_io) {
+  if (io_nf) {
   C rb = m.rho, drb = m.drho, ubx = m.ux, uby = m.uy, ubz = m.uz, usqb = m.usq;
   if (iom & kDirBits) {
     const int k = (int)((iom & kIoletIdBits) >> kIoletShift);
@@ -1049,60 +1147,56 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
   iost[4 * kTile + lane] = ubz;
   iost[5 * kTile + lane] = usqb;
   }
+  Relax<C, false> rx(m, omega);
   // rest population: stays at x
-  {
-    const C g0 = gv(0);
-    Cd::st(P + x, 0, g0 + omega * (geq<0, C>(m.drho, m.rho, m.ux, m.uy, m.uz, m.usq) - g0));
-  }
+  Cd::st(P + x, 0, rx.rest(m, gv(0)));
   chk_count(d.chk, P, P + x, kQ * np, d.err);
-  const bool bounce = !p.elastic;
+  const C keep = C(1) - omega;  // (1 - 1/tau)
+  // coefficients of the wall state (rho, sw u), as rx.wr and rx.l for (rho, u)
+  C wr_w = mul_pin(rx.wr, mul_pin(sw, sw)), l_w = mul_pin(rx.l, sw);
   // Store addresses from a base and a stride (even steps) or a site index
   // (odd steps) the compiler cannot identify with those of the loads (opaque
   // copies): otherwise it keeps the 19 load addresses, or the rows' offsets,
   // live until the stores that reuse them.
-  S* Pst;
-  asm volatile("mov.b64 %0, %1;" : "=l"(Pst) : "l"(P));
+  S* const Pst = opaque_base(P);
   uint32_t xst;
   asm volatile("mov.b32 %0, %1;" : "=r"(xst) : "r"((uint32_t)x));
   unroll<9>([&](auto Pi) {
     constexpr int a = 2 * decltype(Pi)::value + 1, b = a + 1;
     constexpr C w = a <= 6 ? C(1.0 / 18.0) : C(1.0 / 36.0);
-    const C cu = cdot<a, C>(m.ux, m.uy, m.uz);
-    const C wr = m.rho * w;
-    const C wrq = wr * (C(4.5) * cu * cu - m.usq);
-    const C wd = m.drho * w;
-    const C even = wd + wrq;
-    const C odd = C(3) * wr * cu;
-    const C eqa = even + odd, eqb = even - odd;
-    const C ga = gv(a), gb = gv(b);
-    const C sa = ga + omega * (eqa - ga);
-    const C sb = gb + omega * (eqb - gb);
-    // the pair's links leave the fluid at some lane of the tile (warp-uniform)
-    const bool pair_nf = (warp_nf >> a) & 3u;
-    // GZS values of the pair's two directions at a wall: f^eq(rho, sw u) parts
-    C wa = C(0), wb = C(0);
-    if (warp_wall && pair_nf) {
-      const C evw = wd + sw2 * wrq, odw = sw * odd;
-      wa = evw + odw + keep * (ga - eqa);
-      wb = evw - odw + keep * (gb - eqb);
+    if constexpr (a == 7) {  // the first diagonal
+      rx.next();
+      wr_w *= C(0.5);
+      l_w *= C(0.5);
     }
-    // ... and at the site's iolet
-    C ia = C(0), ib = C(0);
-    if (warp_io && pair_nf) {
+    const C cu = cdot<a, C>(m.ux, m.uy, m.uz);
+    C sa, sb, q, ea, eb;
+    rx.pair(cu, gv(a), gv(b), sa, sb, q, ea, eb);
+    const bool nfa = (nf >> a) & 1u, nfb = (nf >> b) & 1u;
+    // What links a and b send on: g*_a, g*_b, into the slot of the link's own
+    // direction at the neighbour - or, when the link leaves the fluid, the
+    // boundary population into the site's slot of the other direction: that of
+    // bounce-back is the same value, those of the GZS form at a wall and at an
+    // iolet, f^eq(rho_b, u_b) + (1 - 1/tau)(g - g^eq), replace it. Nothing is
+    // computed for pairs by which no lane of the tile leaves through a wall (an
+    // iolet): warp-uniform.
+    C va = sa, vb = sb;
+    if ((wall_nf >> a) & 3u) {
+      const C e = fma_pin(wr_w, q, rx.wd);
+      va = nfa ? fma_pin(-keep, eb, fma_pin(-l_w, cu, e)) : va;
+      vb = nfb ? fma_pin(-keep, ea, fma_pin(l_w, cu, e)) : vb;
+    }
+    if ((io_nf >> a) & 3u) {
       const C* iost = area + kAreaIolet * kTile;
       const C rb = iost[0 * kTile + lane], drb = iost[1 * kTile + lane];
       const C cub = cdot<a, C>(iost[2 * kTile + lane], iost[3 * kTile + lane],
                                iost[4 * kTile + lane]);
-      const C evb = w * (drb + rb * (C(4.5) * cub * cub - iost[5 * kTile + lane]));
-      const C odb = w * C(3) * rb * cub;
-      ia = evb + odb + keep * (ga - eqa);
-      ib = evb - odb + keep * (gb - eqb);
+      const C e = mul_pin(w, fma_pin(rb, fma_pin(mul_pin(C(4.5), cub), cub, -iost[5 * kTile + lane]),
+                                     drb));
+      const C lb = mul_pin(C(3), mul_pin(w, rb));
+      va = ((iom >> a) & 1u) ? fma_pin(-keep, eb, fma_pin(-lb, cub, e)) : va;
+      vb = ((iom >> b) & 1u) ? fma_pin(-keep, ea, fma_pin(lb, cub, e)) : vb;
     }
-    // link a (store into direction b's slot when it leaves the fluid) and link b
-    const bool nfa = (nf >> a) & 1u, nfb = (nf >> b) & 1u;
-    const bool ioa = (iom >> a) & 1u, iob = (iom >> b) & 1u;
-    const C va = nfa ? (ioa ? ib : (bounce ? sa : wb)) : sa;
-    const C vb = nfb ? (iob ? ia : (bounce ? sb : wa)) : sb;
     S* pa;
     S* pb;
     if constexpr (ODD) {
@@ -1625,7 +1719,7 @@ __global__ void __launch_bounds__(kStageWarps * 32, kStages <= 2 ? 8 : (kStages 
     const int64_t x = (int64_t)(lane < 16 ? ta[0] : tb[0]) * kTile + 2 * (lane & 15);
     const uint32_t* row = &buf[w][st][lane >> 4][lane & 15];  // row j at + j * 16 words
     using Cd = Codec2<S>;
-    collide2(
+    collide2<true>(
         [&](int j) -> F2 { return Cd::unpack(row[j * (kTile / 2)]); },
         [&](int j) -> F2 { return Cd::unpack(lds_volatile_u32(row + j * (kTile / 2))); }, om,
         d.err, d.err, [&](F2 s0) { Cd::st_al(P + x, s0); },
@@ -1737,10 +1831,11 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
     cp_async_elem(site_row(4) + lane, prof + 2 * d.slot_stride + slot);
   }
   cp_async_commit();
-  // warp-uniform: which boundary states the tile needs at all
-  const bool warp_io = __any_sync(0xFFFFFFFFu, valid && (iom & kDirBits));
-  const bool warp_wall = p.elastic && __any_sync(0xFFFFFFFFu, valid && (smask & kHasWall));
-  const uint32_t warp_nf = __reduce_or_sync(0xFFFFFFFFu, valid ? (smask & kDirBits) : 0u);
+  // the directions by which some lane leaves through an elastic wall, and
+  // through an iolet (warp-uniform)
+  const uint32_t wall_nf =
+      __reduce_or_sync(0xFFFFFFFFu, valid && p.elastic ? (smask & ~iom & kDirBits) : 0u);
+  const uint32_t io_nf = __reduce_or_sync(0xFFFFFFFFu, valid ? (iom & kDirBits) : 0u);
   // sites linked to two or more iolets take the per-link form
   const bool multi = smask & kMultiIolet;
   S* P = static_cast<S*>(d.pop);
@@ -1779,8 +1874,8 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
         ostride = kTile;
       }
       const C r = boundary_fast<S, ODD>(d, p, omega_as<C>(p.omega, p.omega_f), P, x, offp,
-                                        ostride, smask, iom, site, nbr_s, lane, slot, warp_io,
-                                        warp_wall, warp_nf, gsm);
+                                        ostride, smask, iom, site, nbr_s, lane, slot, wall_nf,
+                                        io_nf, gsm);
       if (dr) *dr = r;
     }
     return true;
