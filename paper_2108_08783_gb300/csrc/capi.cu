@@ -87,6 +87,11 @@ struct lbm_ctx {
   // compile-time offset (the parity plus the step within the block)
   int64_t* step_d = nullptr;
   int64_t step_d_for = -1;
+  // small lattices: all steps of a call in one cooperative launch (k_small),
+  // unless a launch knob has been set
+  bool small = false;
+  bool tuned = false;
+  unsigned long long* small_bar = nullptr;
   // tensor map of the populations as a [19][npad] array of 16-bit elements,
   // boxes of 32 x 19 (staged-row bulk kernel), made on first use
   alignas(64) CUtensorMap tmap;
@@ -125,6 +130,9 @@ namespace {
 // Steps per captured graph of a lattice by default: +3 % on the long tube
 // against direct launches (100 gains another 0.1-0.4 %).
 constexpr int64_t kDefaultGraphSteps = 20;
+
+// Steps per launch of the small-lattice kernel (some milliseconds).
+constexpr int64_t kSmallSteps = 1000;
 
 constexpr uint64_t kCkptMagic = 0x314b43504d424cULL;  // "LBMPCK1"
 
@@ -332,6 +340,7 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
   unsigned char* sp = dev_alloc<unsigned char>(c, 3 * S * cb);
   unsigned char* sF = dev_alloc<unsigned char>(c, S * cb);
   double* sK = dev_alloc<double>(c, S);
+  c->small_bar = dev_alloc<unsigned long long>(c, 1);
   double* sdE = dev_alloc<double>(c, S);
   double* sUw = dev_alloc<double>(c, 3 * S);
   lbm::IoletDev* io = dev_alloc<lbm::IoletDev>(c, n_iolets);
@@ -343,7 +352,7 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
   int32_t* mt = L.multi_tiles.empty() ? nullptr : dev_alloc<int32_t>(c, L.multi_tiles.size());
   int32_t* stab = L.seg_tab.empty() ? nullptr : dev_alloc<int32_t>(c, L.seg_tab.size());
   if (!d.pop || !td || !to || !sm || !sio || !sn || !sp || !sF || !sK || !sdE || !sUw ||
-      !io || !err || !c->iolet_off || !c->iolet_sites || !c->partial || !c->red_out ||
+      !io || !err || !c->small_bar || !c->iolet_off || !c->iolet_sites || !c->partial || !c->red_out ||
       (!L.multi_tiles.empty() && !mt) || (!L.seg_tab.empty() && !stab)) {
     g_build_err = "device allocation failed";
     lbm_destroy(c);
@@ -429,12 +438,14 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
     chk(cudaMemsetAsync(sUw, 0, 3 * S * sizeof(double), c->stream));
   }
   chk(cudaMemsetAsync(err, 0, sizeof(int), c->stream));
+  chk(cudaMemsetAsync(c->small_bar, 0, sizeof(unsigned long long), c->stream));
   {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
       c->n_sms = sms;
     cudaGetLastError();
+    c->small = d.n_tiles > 0 && d.n_multi == 0 && d.n_tiles <= lbm::small_tiles(storage, c->n_sms);
   }
   chk(cudaMemsetAsync(d.pop, 0, (size_t)lbm::kQ * d.npad * sz, c->stream));
   if (e != cudaSuccess) {
@@ -583,9 +594,31 @@ lbm::StepParams step_params(const lbm_ctx* c) {
   return p;
 }
 
+// The caller is recording the stream into a graph of its own: steps take the
+// launches that have always been recorded.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
   lbm::StepParams p = step_params(c);
 #ifndef LBM_CHECKED
+  if (c->small && !c->tuned && !diag_last && !c->prof && n_steps > 0 && !capturing(c->stream)) {
+    for (int64_t done = 0; done < n_steps;) {
+      const int64_t m = std::min(n_steps - done, kSmallSteps);
+      p.step = c->step;
+      const int lr = lbm::launch_small(c->storage, c->d, p, m, c->small_bar, c->stream);
+      if (lr != 0) return cuda_fail(c, (cudaError_t)lr, "step kernel");
+      c->step += m;
+      done += m;
+    }
+    return LBM_OK;
+  }
   const int64_t G = c->graph_steps;
   if (G > 0 && n_steps >= G && !diag_last && !c->prof) {
     // whole blocks of G steps as graph replays on the private stream
@@ -807,6 +840,7 @@ int lbm_tune(lbm_ctx* c, int32_t knob, int64_t value) {
   if (!c) return LBM_EINVAL;
   c->err.clear();
   c->gexec_steps = 0;  // a captured step graph holds the old settings: capture again
+  c->tuned = true;     // the launches asked for, whatever the size
   switch (knob) {
     case LBM_TUNE_GRAPH_STEPS:
       if (value < 0 || (value & 1)) return fail(c, LBM_EINVAL, "graph steps must be even and >= 0");
@@ -842,6 +876,9 @@ int lbm_sync(lbm_ctx* c) {
   if (e != cudaSuccess) return cuda_fail(c, e, "lbm_sync flag");
   if (flag) {
     cudaMemsetAsync(c->d.err, 0, sizeof(int), c->stream);
+    // a grid barrier that gave up leaves its counter between two launches
+    if (flag & lbm::kErrTimeout)
+      cudaMemsetAsync(c->small_bar, 0, sizeof(unsigned long long), c->stream);
     cudaStreamSynchronize(c->stream);
     if (flag & lbm::kErrTimeout)
       return fail(c, LBM_ETIMEOUT, "a bounded device wait gave up");

@@ -1766,12 +1766,20 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::one)
 // to one iolet (boundary_fast), 1 the sites linked to two or more iolets (the
 // per-link form, run by k_boundary_multi over the tiles that have such sites),
 // 2 both (the persistent kernel).
-template <class S, bool ODD, int PART = 0>
+// KEEP: the warp updates this one tile step after step (k_small) and everything
+// but the populations is loaded once: `kept` holds the lane's masks, the
+// descriptor, tables and per-site data stay in the warp's areas.
+struct KeptTile {
+  uint32_t have;  // bit 0: loaded; bit 1: the odd steps' neighbour tables too
+  uint32_t smask, iom;
+};
+template <class S, bool ODD, int PART = 0, bool KEEP = false>
 __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepParams& p, int64_t k,
                                               int32_t* dsc, int32_t* nbr_s, uint64_t* bar,
                                               typename Codec<S>::C* gsm, int lane,
                                               uint32_t* bar_phase = nullptr,
-                                              typename Codec<S>::C* dr = nullptr) {
+                                              typename Codec<S>::C* dr = nullptr,
+                                              KeptTile* kept = nullptr) {
   using C = typename Codec<S>::C;
   // a warp that updates tiles in a loop (persistent kernel): lanes that left
   // the previous tile early (padding sites) wait here until every lane is done
@@ -1779,9 +1787,10 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   __syncwarp();
   const int64_t slot = k * kTile + lane;  // boundary tiles lead the launch order
   // per-site data and the descriptor, all in one round trip
-  const uint32_t smask = __ldg(d.slot_mask + slot);
-  const uint32_t iom = __ldg(d.slot_io + slot);
-  if (lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
+  const bool first = !KEEP || !(kept->have & 1u);
+  const uint32_t smask = first ? __ldg(d.slot_mask + slot) : kept->smask;
+  const uint32_t iom = first ? __ldg(d.slot_io + slot) : kept->iom;
+  if (first && lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
   __syncwarp();
   const uint32_t tmask = (uint32_t)dsc[18];
   const bool irr = tmask & kIrregular;
@@ -1793,13 +1802,14 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   // of multi-iolet sites (PART 1, 2) always reads the per-site rows
   const bool seg = ODD && irr && (tmask & kSegmented) && PART == 0;
   const bool stage = ODD && irr && !seg;
-  if (seg) {
+  const bool tables = !KEEP || (ODD && !(kept->have & 2u));
+  if (seg && tables) {
     const int32_t* src = d.seg_tab + k * kSegWords;
     for (int q = lane; q < kSegWords; q += kTile) nbr_s[q] = __ldg(src + q);
   }
   // bar_phase: a warp that stages repeatedly (persistent kernel) keeps one
   // initialised mbarrier and tracks its phase; otherwise it is set up here.
-  if (stage) {
+  if (stage && tables) {
     if (lane == 0 && !bar_phase) mbar_init(bar, 1);
     __syncwarp();
     if (lane == 0) {
@@ -1820,11 +1830,11 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   // type at the start of their rows, kappa c_s^2 (row 1) in FP64.
   double* site = reinterpret_cast<double*>(gsm + kAreaSite * kTile);  // [5][32]
   auto site_row = [&](int r) { return reinterpret_cast<C*>(site + r * kTile); };
-  if (valid && (smask & kHasWall)) {
+  if (first && valid && (smask & kHasWall)) {
     cp_async_elem(site_row(0) + lane, static_cast<const C*>(d.slot_F) + slot);
     cp_async8(site + kTile + lane, d.slot_kappa + slot);
   }
-  if (valid && (smask & kHasInlet)) {
+  if (first && valid && (smask & kHasInlet)) {
     const C* prof = static_cast<const C*>(d.slot_prof);
     cp_async_elem(site_row(2) + lane, prof + slot);
     cp_async_elem(site_row(3) + lane, prof + d.slot_stride + slot);
@@ -1839,7 +1849,12 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   // sites linked to two or more iolets take the per-link form
   const bool multi = smask & kMultiIolet;
   S* P = static_cast<S*>(d.pop);
-  if (stage) {
+  if constexpr (KEEP) {
+    kept->have |= ODD ? 3u : 1u;
+    kept->smask = smask;
+    kept->iom = iom;
+  }
+  if (stage && tables) {
     const uint32_t ph = bar_phase ? *bar_phase : 0u;
     // one decision for the whole warp (lanes could see the limit and the
     // completion in different polls)
@@ -1868,8 +1883,9 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
         offp = nbr_s + kMaxSegments + 18 * q;
       } else if (stage) {
         const uint32_t nfl = smask & kDirBits;
-        for (int i = 1; i < kQ; ++i)
-          if (!((nfl >> i) & 1u)) nbr_s[(i - 1) * kTile + lane] -= (int32_t)x;
+        if (tables)
+          for (int i = 1; i < kQ; ++i)
+            if (!((nfl >> i) & 1u)) nbr_s[(i - 1) * kTile + lane] -= (int32_t)x;
         offp = nbr_s + lane;
         ostride = kTile;
       }
@@ -2180,6 +2196,119 @@ int ensemble_persistent_t(const EnsembleLaunch& e, const StepParams& p, int64_t 
   r = cudaLaunchCooperativeKernel((const void*)k_ensemble_persistent<S>, dim3(blocks),
                                   dim3(kPersistWarps * 32), args, 0, s);
   return (int)r;
+}
+
+// ------------------------------------------------- small lattices, many steps
+// One cooperative launch advances a lattice of few tiles by any number of
+// steps. A step of such a lattice lasts as long as its launches: the 2,226
+// tiles of the R = 12, L = 159 tube took 4.7 us a step in FP32 with two kernels
+// on two streams replayed from a graph, for 1.6 us worth of bytes. Here a warp
+// keeps one tile for the whole launch (tile k goes to warp k / grid of CTA
+// k mod grid, so that the boundary tiles, the first in launch order and the
+// dearest, spread over all SMs): its descriptor, masks, neighbour tables and wall
+// data are loaded once, the populations stay in L2, and the CTAs, one per SM,
+// meet at a barrier between steps: 4.0 us a step, 3.3 on the 416 tiles of
+// the R = 8, L = 64 tube (4.2 from the graph). FP64 gains from the even spread too:
+// its sites cost FP64 issue, and CTAs of four tiles left a third of the SMs
+// without any. With two or more tiles a warp the launched kernels, which fill an
+// SM with more warps, were as fast or faster (5,075 tiles: 6.4 us here, 5.5).
+template <class S>
+struct SmallCfg {
+  static constexpr int warps = 16;  // at most, per CTA: 128 registers a thread
+  using C = typename Codec<S>::C;
+  static constexpr int stage = 18 * kTile * 4, area = BoundaryArea<C>::size * (int)sizeof(C);
+  static constexpr int per_warp = stage + area + 128;  // 128: descriptor and mbarrier
+};
+
+// Grid barrier on a counter that only grows: every launch of a lattice adds a
+// multiple of its (fixed) grid to it, so the first value a CTA reads, before
+// its own first arrival and hence before anyone's second, gives the launch's
+// base; a launch replayed from a caller's graph needs nothing reset. One
+// release-add and an acquiring poll per CTA; bounded spin, false on timeout.
+__device__ __forceinline__ bool small_barrier(unsigned long long* bar, unsigned long long target,
+                                              int* err) {
+  __syncthreads();
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(bar) : "memory");
+    const long long t0 = clock64();
+    for (;;) {
+      unsigned long long v;
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
+      if (v >= target) break;
+      if (clock64() - t0 > kBarrierCycles) {
+        atomicOr(err, kErrTimeout);
+        ok = 0;
+        break;
+      }
+    }
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+template <class S>
+__global__ void __launch_bounds__(SmallCfg<S>::warps * 32, 1)
+    k_small(const DevLattice d, const StepParams p0, int64_t n_steps, unsigned long long* bar) {
+  using C = typename Codec<S>::C;
+  using Cfg = SmallCfg<S>;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  unsigned char* mine = smem + w * Cfg::per_warp;
+  int32_t* stage = reinterpret_cast<int32_t*>(mine);
+  C* area = reinterpret_cast<C*>(mine + Cfg::stage);
+  int32_t* dsc = reinterpret_cast<int32_t*>(mine + Cfg::stage + Cfg::area);
+  uint64_t* mb = reinterpret_cast<uint64_t*>(dsc + 20);
+  __shared__ unsigned long long base;
+  if (lane == 0) mbar_init(mb, 1);
+  if (threadIdx.x == 0) {
+    const unsigned long long v = *static_cast<volatile unsigned long long*>(bar);
+    base = v - v % gridDim.x;
+  }
+  __syncthreads();
+  uint32_t phase = 0;
+  bool ok = true;
+  KeptTile kept{};
+  const int64_t k = blockIdx.x + (int64_t)gridDim.x * w;  // this warp's tile
+  const bool boundary = k < d.n_boundary;
+  if (!boundary && k < d.n_tiles && lane < 20)
+    dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
+  __syncwarp();
+  for (int64_t s = 0; s < n_steps; ++s) {
+    StepParams p = p0;
+    p.step = p0.step + s;
+    p.write_state = s == n_steps - 1 ? 1 : 0;
+    p.step_dev = nullptr;
+    p.diag = 0;
+    const bool odd = p.step & 1;
+    if (boundary) {
+      if (ok)
+        ok = odd ? boundary_tile<S, true, 0, true>(d, p, k, dsc, stage, mb, area, lane, &phase,
+                                                   nullptr, &kept)
+                 : boundary_tile<S, false, 0, true>(d, p, k, dsc, stage, mb, area, lane, &phase,
+                                                    nullptr, &kept);
+    } else if (k < d.n_tiles) {
+      const int64_t x = (int64_t)dsc[19] * kTile + lane;
+      const C om = omega_as<C>(p.omega, p.omega_f);
+      if (odd) bulk_update<S, true>(static_cast<S*>(d.pop), d.npad, x, dsc, om, d.err, d.chk);
+      else bulk_update<S, false>(static_cast<S*>(d.pop), d.npad, x, dsc, om, d.err, d.chk);
+    }
+    if (s + 1 < n_steps && !small_barrier(bar, base + (unsigned long long)(s + 1) * gridDim.x, d.err))
+      return;
+  }
+}
+
+// Warps per CTA and CTAs: a warp per tile, as even over the SMs as they go.
+template <class S>
+int small_t(const DevLattice& d, const StepParams& p, int64_t n_steps, void* bar, cudaStream_t s) {
+  using Cfg = SmallCfg<S>;
+  const int64_t sms = p.n_sms;
+  const int nw = (int)((d.n_tiles + sms - 1) / sms);
+  if (nw < 1 || nw > Cfg::warps) return (int)cudaErrorInvalidValue;  // see small_tiles
+  const unsigned grid = (unsigned)((d.n_tiles + nw - 1) / nw);
+  unsigned long long* b = static_cast<unsigned long long*>(bar);
+  void* args[] = {(void*)&d, (void*)&p, (void*)&n_steps, (void*)&b};
+  return (int)cudaLaunchCooperativeKernel((const void*)k_small<S>, dim3(grid), dim3(nw * 32), args,
+                                          (size_t)nw * Cfg::per_warp, s);
 }
 
 __global__ void k_advance(int64_t* step, int64_t by) { *step += by; }
@@ -2736,6 +2865,32 @@ int launch_ensemble_persistent(int storage, const EnsembleLaunch& e, const StepP
   return dispatch(storage, [&](auto tag) {
     using S = std::remove_pointer_t<decltype(tag)>;
     return ensemble_persistent_t<S>(e, p, n_steps, gs, extra_arrivals, (cudaStream_t)stream);
+  });
+}
+
+int64_t small_tiles(int storage, int n_sms) {
+  int64_t tiles = 0;
+  const int e = dispatch(storage, [&](auto tag) {
+    using S = std::remove_pointer_t<decltype(tag)>;
+    using Cfg = SmallCfg<S>;
+    const int bytes = Cfg::warps * Cfg::per_warp;
+    const int r = (int)cudaFuncSetAttribute(k_small<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            bytes);
+    tiles = (int64_t)n_sms * Cfg::warps;
+    return r;
+  });
+  if (e != 0) {
+    cudaGetLastError();
+    return 0;
+  }
+  return tiles;
+}
+
+int launch_small(int storage, const DevLattice& d, const StepParams& p, int64_t n_steps, void* bar,
+                 void* stream) {
+  return dispatch(storage, [&](auto tag) {
+    using S = std::remove_pointer_t<decltype(tag)>;
+    return small_t<S>(d, p, n_steps, bar, (cudaStream_t)stream);
   });
 }
 

@@ -281,6 +281,13 @@ struct GridSync {
 int launch_ensemble_persistent(int storage, const EnsembleLaunch& e, const StepParams& p,
                                int64_t n_steps, GridSync* sync, int extra_arrivals,
                                void* stream);
+// Small lattices: n_steps >= 1 steps in one cooperative launch. `bar` is a
+// zeroed device counter (8 bytes) of the lattice's own. small_tiles: the most
+// tiles it is used for on a device of n_sms SMs (0: not available; call with
+// the device current before the first launch).
+int64_t small_tiles(int storage, int n_sms);
+int launch_small(int storage, const DevLattice& d, const StepParams& p, int64_t n_steps, void* bar,
+                 void* stream);
 int launch_advance(int64_t* step_dev, int64_t by, void* stream);
 int launch_set_step(int64_t* step_dev, int64_t value, void* stream);
 int launch_init(int storage, const DevLattice& d, const double* rho, const double* u,
