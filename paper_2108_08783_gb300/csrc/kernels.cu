@@ -975,13 +975,21 @@ __device__ __forceinline__ void boundary_load(const S* P, int64_t np, int64_t x,
 }
 
 // Per-warp shared-memory area of the boundary kernels, in compute-type units:
-// rows 0..18 the parked populations g, rows 19..24 the lanes' iolet states,
-// then [5][32] doubles of per-site data (F, kappa/3, inlet profile p0, ps, pc).
-template <class C>
+// with PARK rows 0..18 for parked populations g, then 6 rows of the lanes' iolet
+// states, then [5][32] doubles of per-site data (F, kappa/3, inlet profile p0,
+// ps, pc).  What the areas of an SM do not take is L1, which serves the odd
+// steps' gathers: FP32-compute kernels, which keep g in registers, leave out the
+// parked rows (27 -> 18 KB a CTA; the tree's
+// FP32 step 141.2 -> 139.8 us).
+template <class C, bool PARK>
 struct BoundaryArea {
-  static constexpr int size = 25 * kTile + 5 * kTile * (int)(sizeof(double) / sizeof(C));
+  static constexpr int iolet = PARK ? 19 : 0;  // first row of the iolet states
+  static constexpr int site = iolet + 6;       // first row of the per-site doubles
+  static constexpr int size = site * kTile + 5 * kTile * (int)(sizeof(double) / sizeof(C));
 };
-constexpr int kAreaIolet = 19;  // first row of the iolet states
+// The layout boundary_tile uses: parked rows for FP64 and the per-link form.
+template <class C, int PART>
+using TileArea = BoundaryArea<C, std::is_same<C, double>::value || PART != 0>;
 
 // Fused diagnostics: the momentum rho u of a site with iolet links, at its
 // place among the lanes of the tiles that have such sites, for the fluxes.
@@ -993,7 +1001,6 @@ __device__ __forceinline__ void diag_momentum(const DevLattice& d, int64_t slot,
   d.diag_j[js + q] = (double)(m.rho * m.uy);
   d.diag_j[2 * js + q] = (double)(m.rho * m.uz);
 }
-constexpr int kAreaSite = 25;   // first row (compute-type units) of the per-site doubles
 
 // Update of a boundary site whose iolet links (if any) all lead to one iolet,
 // without branches that differ between lanes: every direction does one load
@@ -1025,7 +1032,7 @@ constexpr bool opposites_adjacent() {
 }
 static_assert(opposites_adjacent(), "opposite directions must be adjacent");
 
-template <class S, bool ODD>
+template <class S, bool ODD, class AREA>
 __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& d,
                                                               const StepParams& p,
                                               typename Codec<S>::C omega, S* P, int64_t x,
@@ -1139,7 +1146,7 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
       outlet_density(io, rb, drb);
     }
   }
-  C* iost = area + kAreaIolet * kTile;
+  C* iost = area + AREA::iolet * kTile;
   iost[0 * kTile + lane] = rb;
   iost[1 * kTile + lane] = drb;
   iost[2 * kTile + lane] = ubx;
@@ -1187,7 +1194,7 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
       vb = nfb ? fma_pin(-keep, ea, fma_pin(l_w, cu, e)) : vb;
     }
     if ((io_nf >> a) & 3u) {
-      const C* iost = area + kAreaIolet * kTile;
+      const C* iost = area + AREA::iolet * kTile;
       const C rb = iost[0 * kTile + lane], drb = iost[1 * kTile + lane];
       const C cub = cdot<a, C>(iost[2 * kTile + lane], iost[3 * kTile + lane],
                                iost[4 * kTile + lane]);
@@ -1752,12 +1759,11 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::one)
   else bulk_tile<S, ODD>(d, p, k, desc_s[w], lane);
 }
 
-// Resident CTAs (4 warps) per SM requested of the boundary kernel: 7, i.e. 73
-// registers, measured on the long tube and the depth-6 tree against 6, 8 and
-// 10 (tree FP32 +8 %, tube FP32 +3 %, FP16S +1-3 % over 8, whose 64 registers
-// spill on odd steps).
+// Resident CTAs (4 warps) per SM requested of the boundary kernel: 8, i.e. 64
+// registers, against 7 (72) and 6: depth-6 tree of root radius 36 FP32 138.5,
+// 139.8, 143.1 us a step, FP16 106.9, 108.7, 112.6; long tube within 0.1 %.
 #ifndef LBM_BOUNDARY_MINB
-#define LBM_BOUNDARY_MINB 7
+#define LBM_BOUNDARY_MINB 8
 #endif
 // Boundary tile at launch position k (whole warp); nbr_s, bar: the warp's
 // staging area (18 rows of per-site neighbours) and mbarrier; dsc: its
@@ -1781,6 +1787,7 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
                                               typename Codec<S>::C* dr = nullptr,
                                               KeptTile* kept = nullptr) {
   using C = typename Codec<S>::C;
+  using Area = TileArea<C, PART>;
   // a warp that updates tiles in a loop (persistent kernel): lanes that left
   // the previous tile early (padding sites) wait here until every lane is done
   // with its descriptor, segment table and staged rows
@@ -1824,11 +1831,11 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   }
   const bool valid = smask & kValid;
   // per-site wall and inlet data (F, kappa/3, inlet profile p0, ps, pc) into
-  // the warp's area (from row kAreaSite), copied asynchronously so that no register
+  // the warp's area (from row Area::site), copied asynchronously so that no register
   // holds them while the populations load
   // Rows of 32 doubles: F (row 0) and p0, ps, pc (rows 2-4) in the compute
   // type at the start of their rows, kappa c_s^2 (row 1) in FP64.
-  double* site = reinterpret_cast<double*>(gsm + kAreaSite * kTile);  // [5][32]
+  double* site = reinterpret_cast<double*>(gsm + Area::site * kTile);  // [5][32]
   auto site_row = [&](int r) { return reinterpret_cast<C*>(site + r * kTile); };
   if (first && valid && (smask & kHasWall)) {
     cp_async_elem(site_row(0) + lane, static_cast<const C*>(d.slot_F) + slot);
@@ -1889,7 +1896,7 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
         offp = nbr_s + lane;
         ostride = kTile;
       }
-      const C r = boundary_fast<S, ODD>(d, p, omega_as<C>(p.omega, p.omega_f), P, x, offp,
+      const C r = boundary_fast<S, ODD, Area>(d, p, omega_as<C>(p.omega, p.omega_f), P, x, offp,
                                         ostride, smask, iom, site, nbr_s, lane, slot, wall_nf,
                                         io_nf, gsm);
       if (dr) *dr = r;
@@ -1922,7 +1929,7 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_
   p.diag = DIAG;  // a compile-time constant for the tile code
   using C = typename Codec<S>::C;
   __shared__ __align__(128) int32_t stage[kBoundaryWarps][18 * kTile];
-  __shared__ __align__(16) C gs[kBoundaryWarps][BoundaryArea<C>::size];
+  __shared__ __align__(16) C gs[kBoundaryWarps][TileArea<C, 0>::size];
   __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1946,7 +1953,7 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32)
   p.diag = DIAG;
   using C = typename Codec<S>::C;
   __shared__ __align__(128) int32_t stage[kBoundaryWarps][18 * kTile];
-  __shared__ __align__(16) C gs[kBoundaryWarps][BoundaryArea<C>::size];
+  __shared__ __align__(16) C gs[kBoundaryWarps][TileArea<C, 1>::size];
   __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2022,7 +2029,7 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_
     k_boundary_ens(const EnsembleLaunch e, const StepParams p) {
   using C = typename Codec<S>::C;
   __shared__ __align__(128) int32_t stage[kBoundaryWarps][18 * kTile];
-  __shared__ __align__(16) C gs[kBoundaryWarps][BoundaryArea<C>::size];
+  __shared__ __align__(16) C gs[kBoundaryWarps][TileArea<C, 0>::size];
   __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2108,7 +2115,7 @@ __global__ void __launch_bounds__(kPersistWarps * 32, sizeof(S) == 8 ? 1 : 4)
                           GridSync* gs, unsigned expected, int chunk) {
   using C = typename Codec<S>::C;
   __shared__ __align__(128) int32_t stage[kPersistWarps][18 * kTile];
-  __shared__ __align__(16) C gsm[kPersistWarps][BoundaryArea<C>::size];
+  __shared__ __align__(16) C gsm[kPersistWarps][TileArea<C, 2>::size];
   __shared__ __align__(16) int32_t desc_s[kPersistWarps][20];
   __shared__ uint64_t bars[kPersistWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2216,7 +2223,7 @@ template <class S>
 struct SmallCfg {
   static constexpr int warps = 16;  // at most, per CTA: 128 registers a thread
   using C = typename Codec<S>::C;
-  static constexpr int stage = 18 * kTile * 4, area = BoundaryArea<C>::size * (int)sizeof(C);
+  static constexpr int stage = 18 * kTile * 4, area = TileArea<C, 0>::size * (int)sizeof(C);
   static constexpr int per_warp = stage + area + 128;  // 128: descriptor and mbarrier
 };
 
