@@ -1239,6 +1239,8 @@ struct lbm_ensemble {
   std::vector<void*> owned;       // device buffers (member 0's allocator)
   lbm::MemberDev* mem_d = nullptr;
   lbm::TileRef* map_d = nullptr;  // tile maps: bulk tiles, then boundary tiles
+  lbm::EnsDesc* desc_d = nullptr;  // bulk tile descriptors, members padded to even numbers
+  int64_t n_desc = 0;
   int64_t n_bulk = 0, n_boundary = 0;  // tiles of all members
   int64_t* step_d = nullptr;      // device step counter of captured graphs
   std::vector<int32_t> order;     // schedule: member order in the launch numbering
@@ -1326,9 +1328,35 @@ int ens_upload(lbm_ensemble* e) {
   e->launch.n_multi_members = (int32_t)e->multi_host.size();
   e->launch.mem = e->mem_d;
   e->launch.n_members = n;
+  e->launch.desc = e->desc_d;
+  e->launch.n_desc = e->n_desc;
   e->launch.n_bulk_tiles = e->n_bulk;
   e->launch.n_boundary_tiles = e->n_boundary;
   ens_drop_graph(e);
+  return LBM_OK;
+}
+
+// The bulk tiles' descriptors in schedule order, from the members' launch lists
+// (after ens_upload: the kernel reads the member table).
+int ens_descs(lbm_ensemble* e) {
+  if (e->n_desc == 0) return LBM_OK;
+  std::vector<lbm::TileRef> map;
+  map.reserve((size_t)e->n_desc);
+  for (int q = 0; q < (int)e->members.size(); ++q) {
+    const lbm_ctx* c = e->members[e->order[q]];
+    for (int64_t k = c->d.n_boundary; k < c->d.n_tiles; ++k) map.push_back(lbm::TileRef{q, (int32_t)k});
+    if (map.size() & 1) map.push_back(lbm::TileRef{q, -1});
+  }
+  Temp t(e->members[0], map.size() * sizeof(lbm::TileRef));
+  if (!t.p) return ens_fail(e, LBM_ENOMEM, "ensemble descriptors: allocation");
+  cudaError_t r = cudaMemcpyAsync(t.p, map.data(), map.size() * sizeof(lbm::TileRef),
+                                  cudaMemcpyHostToDevice, e->stream);
+  if (r == cudaSuccess)
+    r = (cudaError_t)lbm::launch_ens_desc(e->storage, e->mem_d, static_cast<lbm::TileRef*>(t.p),
+                                          (int64_t)map.size(), e->desc_d, e->stream);
+  const cudaError_t r2 = cudaStreamSynchronize(e->stream);  // the maps are temporaries
+  if (r == cudaSuccess) r = r2;
+  if (r != cudaSuccess) return ens_cuda(e, r, "ensemble descriptors");
   return LBM_OK;
 }
 
@@ -1366,8 +1394,11 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
   if (!e) return LBM_ENOMEM;
   e->members.assign(members, members + n);
   e->storage = members[0]->storage;
-  e->prefetch = default_prefetch(e->storage);
-  e->bulk_sites = default_bulk_sites(e->storage);
+  // measured on 48 tubes (12.5 M sites): two sites per lane and no prefetch for
+  // FP32 too (350 us a step; one site per lane 369 with a prefetch of 4,096
+  // tiles, 372 without; two sites and 2,048 tiles 365)
+  e->prefetch = 0;
+  e->bulk_sites = e->storage == LBM_F64 ? 1 : 2;
   for (lbm_ctx* c : e->members)
     if (std::find(e->member_streams.begin(), e->member_streams.end(), c->stream) ==
         e->member_streams.end())
@@ -1394,19 +1425,25 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
   for (lbm_ctx* c : e->members) {
     e->n_bulk += c->d.n_tiles - c->d.n_boundary;
     e->n_boundary += c->d.n_boundary;
+    e->n_desc += (c->d.n_tiles - c->d.n_boundary + 1) / 2 * 2;
   }
   e->mem_d = static_cast<lbm::MemberDev*>(alloc(n * sizeof(lbm::MemberDev)));
   e->map_d = static_cast<lbm::TileRef*>(
       alloc(std::max<int64_t>(1, e->n_bulk + e->n_boundary) * sizeof(lbm::TileRef)));
+  e->desc_d = static_cast<lbm::EnsDesc*>(
+      alloc(std::max<int64_t>(1, e->n_desc) * sizeof(lbm::EnsDesc)));
   e->step_d = static_cast<int64_t*>(alloc(sizeof(int64_t)));
   e->sync_d = static_cast<lbm::GridSync*>(alloc(sizeof(lbm::GridSync)));
-  if (!e->mem_d || !e->map_d || !e->step_d || !e->sync_d) {
+  if (!e->mem_d || !e->map_d || !e->desc_d || !e->step_d || !e->sync_d) {
     lbm_ensemble_destroy(e);
     return LBM_ENOMEM;
   }
-  if (ens_maps(e) != LBM_OK || ens_upload(e) != LBM_OK) {
+  int rc = ens_maps(e);
+  if (rc == LBM_OK) rc = ens_upload(e);
+  if (rc == LBM_OK) rc = ens_descs(e);
+  if (rc != LBM_OK) {
     lbm_ensemble_destroy(e);
-    return LBM_ECUDA;
+    return rc;
   }
   *out = e;
   return LBM_OK;
@@ -1431,8 +1468,10 @@ int lbm_ensemble_tune(lbm_ensemble* e, int32_t knob, int64_t value) {
       } else if (value != 0) {
         return ens_fail(e, LBM_EINVAL, "schedule must be 0 (given order) or 1 (largest first)");
       }
-      if (ens_maps(e) != LBM_OK) return LBM_ECUDA;
-      return ens_upload(e);
+      int rc = ens_maps(e);
+      if (rc == LBM_OK) rc = ens_upload(e);
+      if (rc == LBM_OK) rc = ens_descs(e);
+      return rc;
     }
     case LBM_TUNE_GRAPH_STEPS:
       if (value < 0 || (value & 1)) return ens_fail(e, LBM_EINVAL, "graph steps must be even");

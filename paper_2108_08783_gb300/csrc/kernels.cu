@@ -503,12 +503,16 @@ constexpr bool kChecked = true;
 #else
 constexpr bool kChecked = false;
 #endif
-template <class S>
-__device__ __forceinline__ void chk_count(int* chk, const S* P0, const S* p, int64_t lim, int* err) {
+// Where a site update flags its errors: a lattice's own word, or that of an
+// ensemble's member, looked up only when there is something to flag.
+__device__ __forceinline__ int* err_word(int* err) { return err; }
+__device__ __forceinline__ int* err_word(const MemberDev* m) { return m->d.err; }
+template <class S, class E>
+__device__ __forceinline__ void chk_count(int* chk, const S* P0, const S* p, int64_t lim, E err) {
   if constexpr (kChecked) {
     if (!chk) return;
     const int64_t i = p - P0;
-    if (i < 0 || i >= lim) atomicOr(err, kErrCheck);
+    if (i < 0 || i >= lim) atomicOr(err_word(err), kErrCheck);
     else atomicAdd(chk + i, 1);
   }
 }
@@ -532,15 +536,31 @@ __device__ __forceinline__ S* opaque_base(S* p) {
   return q;
 }
 
+// The base and row length the stores of an update use.  A single lattice's row
+// length is a kernel parameter, so the 19 row offsets live in uniform
+// registers; a member's (E = const MemberDev*) is loaded, and without opaque
+// copies of both the compiler keeps 19 64-bit products from the loads to the
+// stores.
+template <class S, bool ODD, class E>
+struct StoreBase {
+  S* q;
+  int64_t np;
+  __device__ __forceinline__ StoreBase(S* p, int64_t n) : q(p), np(n) {
+    constexpr bool member = !std::is_same<E, int*>::value;
+    if constexpr (member || !ODD) q = opaque_base(p);
+    if constexpr (member) asm volatile("mov.b64 %0, %1;" : "=l"(np) : "l"(n));
+  }
+};
+
 // Branch-free update of a site whose 18 links are fluid.
 // Returns the site's rho - 1 (for the fused mass diagnostic).  With SLOT the
 // whole warp (every lane updating a site) adds the lanes' rho - 1 as soon as
 // the moments are formed and lane 0 writes the sum to *slot, so nothing of it
 // stays live through the stores.
-template <class S, bool ODD, bool SLOT = false>
+template <class S, bool ODD, bool SLOT = false, class E = int*>
 __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, int64_t x,
                                                             const int32_t* dsc,
-                                                            typename Codec<S>::C omega, int* err,
+                                                            typename Codec<S>::C omega, E err,
                                                             int* chk, double* slot = nullptr) {
   using Cd = Codec<S>;
   using C = typename Cd::C;
@@ -556,10 +576,10 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
     const C sum = warp_sum(m.drho);
     if ((threadIdx.x & 31) == 0) *slot = (double)sum;
   }
-  if (unstable(m.rho)) atomicOr(err, kErrUnstable);
+  if (unstable(m.rho)) atomicOr(err_word(err), kErrUnstable);
   Relax<C, !std::is_same<S, float>::value> rx(m, omega);
-  S* const Q = ODD ? P : opaque_base(P);
-  Cd::st(Q + x, 0, rx.rest(m, g[0]));
+  const StoreBase<S, ODD, E> B(P, np);
+  Cd::st(B.q + x, 0, rx.rest(m, g[0]));
   chk_count(chk, P, P + x, kQ * np, err);
   unroll<9>([&](auto Pi) {
     constexpr int a = 2 * decltype(Pi)::value + 1, b = a + 1;
@@ -570,15 +590,15 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
       // The store to (x + c_a, a) hits the address the load of direction
       // opp(a) used; re-reading the offset from shared memory keeps the
       // compiler from holding all 18 64-bit addresses live across the update.
-      S* pa = P + a * np + x + lds_volatile(dsc + a - 1);
-      S* pb = P + b * np + x + lds_volatile(dsc + b - 1);
+      S* pa = B.q + a * B.np + x + lds_volatile(dsc + a - 1);
+      S* pb = B.q + b * B.np + x + lds_volatile(dsc + b - 1);
       Cd::st(pa, a, sa);
       Cd::st(pb, b, sb);
       chk_count(chk, P, pa, kQ * np, err);
       chk_count(chk, P, pb, kQ * np, err);
     } else {
-      Cd::st(Q + b * np + x, a, sa);
-      Cd::st(Q + a * np + x, b, sb);
+      Cd::st(B.q + b * B.np + x, a, sa);
+      Cd::st(B.q + a * B.np + x, b, sb);
       chk_count(chk, P, P + b * np + x, kQ * np, err);
       chk_count(chk, P, P + a * np + x, kQ * np, err);
     }
@@ -716,9 +736,8 @@ struct Codec2<__nv_bfloat16> {
   }
 };
 
-template <class S>
-__device__ __forceinline__ void chk_count2(int* chk, const S* P0, const S* p, int64_t lim,
-                                           int* err) {
+template <class S, class E>
+__device__ __forceinline__ void chk_count2(int* chk, const S* P0, const S* p, int64_t lim, E err) {
   chk_count(chk, P0, p, lim, err);
   chk_count(chk, P0, p + 1, lim, err);
 }
@@ -728,9 +747,9 @@ __device__ __forceinline__ void chk_count2(int* chk, const S* P0, const S* p, in
 // for the relaxation (the 16-bit paths unpack them twice from packed words
 // rather than hold 38 floats); store0(g*_0) receives the rest population and
 // store<a, b>(g*_a, g*_b) those of each opposite pair (a odd, b = a + 1).
-template <bool SCALED, class GetM, class GetP, class St0, class St>
-__device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, int* err_lo,
-                                       int* err_hi, St0&& store0, St&& store) {
+template <bool SCALED, class E, class GetM, class GetP, class St0, class St>
+__device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, E err, St0&& store0,
+                                       St&& store) {
   // Eqs. (Density), (Momentum), grouped as in moments()
   F2 g[kQ];
   unroll<kQ>([&](auto J) {
@@ -751,8 +770,7 @@ __device__ __forceinline__ F2 collide2(GetM&& gm, GetP&& gp, F2 omega, int* err_
   const F2 rho = add2(bc2(1.0f), drho);
   float r0, r1;
   split2(rho, r0, r1);
-  if (unstable(r0)) atomicOr(err_lo, kErrUnstable);
-  if (unstable(r1)) atomicOr(err_hi, kErrUnstable);
+  if (unstable(r0) || unstable(r1)) atomicOr(err_word(err), kErrUnstable);
   float d0, d1;
   split2(drho, d0, d1);
   const F2 inv = mk2(inv_one_plus(d0, r0, rcp_estimate(r0)), inv_one_plus(d1, r1, rcp_estimate(r1)));
@@ -824,9 +842,9 @@ __device__ __forceinline__ float sum2(F2 a) {
 // Branch-free update of the sites x, x + 1 (x even) whose 18 links are fluid,
 // both with the neighbour offsets dsc: one address per direction for both
 // sites, packed loads and stores where the offset is even.
-template <class S, bool ODD>
+template <class S, bool ODD, class E>
 __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const int32_t* dsc,
-                                              float omega, int* err, int* chk) {
+                                              float omega, E err, int* chk) {
   using Cd = Codec2<S>;
   constexpr bool kPacked = sizeof(S) == 2;
   F2 g[kPacked ? 1 : kQ];
@@ -854,19 +872,19 @@ __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const
     if constexpr (kPacked) return Cd::unpack(opaque(r[j]));
     else return g[j];
   };
-  S* const Q = ODD ? P : opaque_base(P);
-  return sum2(collide2<sizeof(S) == 2>(
-      gm, gp, bc2(omega), err, err,
+  const StoreBase<S, ODD, E> B(P, np);
+  return sum2(collide2<sizeof(S) == 2, E>(
+      gm, gp, bc2(omega), err,
       [&](F2 s0) {
-        Cd::st_al(Q + x, s0);
+        Cd::st_al(B.q + x, s0);
         chk_count2(chk, P, P + x, kQ * np, err);
       },
       [&](auto A, F2 sa, F2 sb) {
         constexpr int a = decltype(A)::value, b = a + 1;
         if constexpr (ODD) {
           const int32_t da = lds_volatile(dsc + a - 1), db = lds_volatile(dsc + b - 1);
-          S* pa = P + a * np + x + da;
-          S* pb = P + b * np + x + db;
+          S* pa = B.q + a * B.np + x + da;
+          S* pb = B.q + b * B.np + x + db;
           if (da & 1) Cd::st_un(pa, sa);
           else Cd::st_al(pa, sa);
           if (db & 1) Cd::st_un(pb, sb);
@@ -874,8 +892,8 @@ __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const
           chk_count2(chk, P, pa, kQ * np, err);
           chk_count2(chk, P, pb, kQ * np, err);
         } else {
-          Cd::st_al(Q + b * np + x, sa);
-          Cd::st_al(Q + a * np + x, sb);
+          Cd::st_al(B.q + b * B.np + x, sa);
+          Cd::st_al(B.q + a * B.np + x, sb);
           chk_count2(chk, P, P + b * np + x, kQ * np, err);
           chk_count2(chk, P, P + a * np + x, kQ * np, err);
         }
@@ -887,10 +905,10 @@ __device__ __forceinline__ float bulk_update2(S* P, int64_t np, int64_t x, const
 // SAME: the second tile directly follows the first with the same offsets, so
 // each of its addresses is the first tile's plus one tile (an immediate
 // offset, no second address).
-template <class S, bool ODD, bool SAME>
+template <class S, bool ODD, bool SAME, class E>
 __device__ __forceinline__ float bulk_update2v(S* P, int64_t np, int64_t xa, int64_t xb,
                                               const int32_t* da, const int32_t* db, float omega,
-                                              int* err, int* chk) {
+                                              E err, int* chk) {
   using Cd = Codec<S>;
   constexpr bool kPacked = sizeof(S) == 2;
   F2 g[kPacked ? 1 : kQ];
@@ -925,23 +943,24 @@ __device__ __forceinline__ float bulk_update2v(S* P, int64_t np, int64_t xa, int
     chk_count(chk, P, pa, kQ * np, err);
     chk_count(chk, P, pb, kQ * np, err);
   };
-  return sum2(collide2<sizeof(S) == 2>(
-      gm, gp, bc2(omega), err, err,
-      [&](F2 s0) { put(P + xa, SAME ? P + xa + kTile : P + xb, s0, 0); },
+  const StoreBase<S, ODD, E> B(P, np);
+  return sum2(collide2<sizeof(S) == 2, E>(
+      gm, gp, bc2(omega), err,
+      [&](F2 s0) { put(B.q + xa, SAME ? B.q + xa + kTile : B.q + xb, s0, 0); },
       [&](auto A, F2 sa, F2 sb) {
         constexpr int i = decltype(A)::value, k = i + 1;  // the pair (i, k = opp i)
         if constexpr (ODD) {
-          S* pi = P + i * np + xa + lds_volatile(da + i - 1);
-          S* pk = P + k * np + xa + lds_volatile(da + k - 1);
-          S* qi = SAME ? pi + kTile : P + i * np + xb + lds_volatile(db + i - 1);
-          S* qk = SAME ? pk + kTile : P + k * np + xb + lds_volatile(db + k - 1);
+          S* pi = B.q + i * B.np + xa + lds_volatile(da + i - 1);
+          S* pk = B.q + k * B.np + xa + lds_volatile(da + k - 1);
+          S* qi = SAME ? pi + kTile : B.q + i * B.np + xb + lds_volatile(db + i - 1);
+          S* qk = SAME ? pk + kTile : B.q + k * B.np + xb + lds_volatile(db + k - 1);
           put(pi, qi, sa, i);
           put(pk, qk, sb, k);
         } else {
-          S* pk = P + k * np + xa;
-          S* pi = P + i * np + xa;
-          put(pk, SAME ? pk + kTile : P + k * np + xb, sa, i);
-          put(pi, SAME ? pi + kTile : P + i * np + xb, sb, k);
+          S* pk = B.q + k * B.np + xa;
+          S* pi = B.q + i * B.np + xa;
+          put(pk, SAME ? pk + kTile : B.q + k * B.np + xb, sa, i);
+          put(pi, SAME ? pi + kTile : B.q + i * B.np + xb, sb, k);
         }
       }));
 }
@@ -1445,17 +1464,20 @@ struct BulkMinBlocks {
   static constexpr int two_ctas = sizeof(S) == 2 ? LBM_BULK2_MINB16 : LBM_BULK2_MINB;
   static constexpr int two = two_ctas * 4 / W < 1 ? 1 : two_ctas * 4 / W;
 };
-// The ensemble kernels hold each member's pointers and strides in registers
+// The ensemble kernels hold the member's pointer and row length in registers
 // (a single lattice reads them from the kernel parameters), so they get their
-// own register budgets, measured on the 256-tube ensemble: 80 registers for the
-// one-site bulk kernel (FP32 +14 % over 64, which spill), 128 for the two-site
-// bulk kernel (FP16S +11 % over 80), 72 for the boundary kernel (FP16S +7 %
-// over 80, +2 % over 64).
+// own register budgets, measured on 48 tubes of the ensemble (12.5 M sites):
+// one site per lane 64 (FP32, prefetch of 4,096 tiles: 369 us a step, 375 at
+// 72); two sites 80 for FP32 (350 us a step, 355 at 72, 366 at 64, which
+// spill) and 64 for 16-bit storage (262 us, 265 at 72, 267 at 80).
 #ifndef LBM_ENS_BULK_MINB
-#define LBM_ENS_BULK_MINB 6
+#define LBM_ENS_BULK_MINB 8
 #endif
 #ifndef LBM_ENS_BULK2_MINB
-#define LBM_ENS_BULK2_MINB 4
+#define LBM_ENS_BULK2_MINB 6
+#endif
+#ifndef LBM_ENS_BULK2_MINB16
+#define LBM_ENS_BULK2_MINB16 8
 #endif
 #ifndef LBM_ENS_BOUNDARY_MINB
 #define LBM_ENS_BOUNDARY_MINB 7
@@ -1463,7 +1485,8 @@ struct BulkMinBlocks {
 template <class S, int W>
 struct EnsBulkMinBlocks {
   static constexpr int one = sizeof(S) == 8 ? 16 / W : LBM_ENS_BULK_MINB * 4 / W;
-  static constexpr int two = LBM_ENS_BULK2_MINB * 4 / W < 1 ? 1 : LBM_ENS_BULK2_MINB * 4 / W;
+  static constexpr int two =
+      (sizeof(S) == 2 ? LBM_ENS_BULK2_MINB16 : LBM_ENS_BULK2_MINB) * 4 / W;
 };
 #ifndef LBM_BOUNDARY_WARPS
 #define LBM_BOUNDARY_WARPS 4
@@ -1518,8 +1541,7 @@ __device__ __forceinline__ typename Codec<S>::C bulk_tile(const DevLattice& d,
 }
 
 
-// The fields of a lattice the bulk kernels read (a member of an ensemble is
-// read field by field from its device table, not copied whole).
+// The fields of a lattice the bulk kernels read.
 struct BulkView {
   void* pop;
   const LaunchDesc* launch;
@@ -1531,78 +1553,60 @@ __device__ __forceinline__ BulkView bulk_view(const DevLattice& d) {
   return BulkView{d.pop, d.launch, d.err, d.chk, d.npad, d.n, d.n_tiles};
 }
 
-// Two bulk tiles per warp, two sites per lane (FP32 and 16-bit storage): tile
-// A at launch position kA of lattice dA and, when `two`, tile B at launch
-// position kB of lattice dB (the same lattice, or another member of an
-// ensemble); omA, omB their relaxation rates; dsc2: the warp's two 20-word
-// descriptor areas.
+// Two bulk tiles per warp, two sites per lane (FP32 and 16-bit storage): the
+// tiles at launch positions k0 and, when `two`, k0 + 1; dsc2: the warp's two
+// 20-word descriptor areas.
 //   VERT = false: lanes 0..15 take tile A, lanes 16..31 tile B, lane l the
 //     z-adjacent sites 2 (l mod 16), 2 (l mod 16) + 1 of its tile (packed words);
 //   VERT = true: lane l takes site l of both tiles (scalar accesses; one
-//     address for both when B directly follows A in the same lattice with the
-//     same offsets).
+//     address for both when B directly follows A with the same offsets).
 // A site without a partner takes the single-site update.
 template <class S, bool ODD, bool VERT>
-__device__ __forceinline__ float bulk_pair_warp(const BulkView& dA, int64_t kA, float omA,
-                                               const BulkView& dB, int64_t kB, float omB,
-                                               bool two, bool one_lattice, int64_t prefetch,
-                                               int32_t (*dsc2)[20], int lane) {
+__device__ __forceinline__ float bulk_pair_warp(const BulkView& d, int64_t k0, float om, bool two,
+                                               int64_t prefetch, int32_t (*dsc2)[20], int lane) {
   if (lane < 20) {
-    dsc2[0][lane] = __ldg(reinterpret_cast<const int32_t*>(dA.launch + kA) + lane);
-    if (two) dsc2[1][lane] = __ldg(reinterpret_cast<const int32_t*>(dB.launch + kB) + lane);
+    dsc2[0][lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k0) + lane);
+    if (two) dsc2[1][lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k0 + 1) + lane);
   }
   if (prefetch > 0 && lane < kQ) {
-    if (kA + prefetch < dA.n_tiles) {
-      const int64_t tp = __ldg(&dA.launch[kA + prefetch].tile);
-      bulk_prefetch_l2(static_cast<const S*>(dA.pop) + lane * dA.npad + tp * kTile,
-                       kTile * sizeof(S));
-    }
-    if (two && kB + prefetch < dB.n_tiles) {
-      const int64_t tp = __ldg(&dB.launch[kB + prefetch].tile);
-      bulk_prefetch_l2(static_cast<const S*>(dB.pop) + lane * dB.npad + tp * kTile,
+    for (int64_t k = k0 + prefetch; k < k0 + prefetch + 2 && k < d.n_tiles; ++k) {
+      const int64_t tp = __ldg(&d.launch[k].tile);
+      bulk_prefetch_l2(static_cast<const S*>(d.pop) + lane * d.npad + tp * kTile,
                        kTile * sizeof(S));
     }
   }
   __syncwarp();
+  S* P = static_cast<S*>(d.pop);
   if constexpr (!VERT) {
     const int half = lane >> 4;
     if (half && !two) return 0.0f;
-    // this half's lattice, field by field (no reference chosen at run time)
-    S* P = static_cast<S*>(half ? dB.pop : dA.pop);
-    const int64_t np = half ? dB.npad : dA.npad, n = half ? dB.n : dA.n;
-    int* err = half ? dB.err : dA.err;
-    int* chk = half ? dB.chk : dA.chk;
     const int32_t* dsc = dsc2[half];
     const int64_t x = (int64_t)dsc[19] * kTile + 2 * (lane & 15);
-    if (x >= n) return 0.0f;
+    if (x >= d.n) return 0.0f;
     if constexpr (kChecked && ODD) {
       bool ok = true;
-      for (int o = 0; o < 18; ++o) ok = chk_site(x + dsc[o], n, err) && ok;
-      if (x + 1 < n)
-        for (int o = 0; o < 18; ++o) ok = chk_site(x + 1 + dsc[o], n, err) && ok;
+      for (int o = 0; o < 18; ++o) ok = chk_site(x + dsc[o], d.n, d.err) && ok;
+      if (x + 1 < d.n)
+        for (int o = 0; o < 18; ++o) ok = chk_site(x + 1 + dsc[o], d.n, d.err) && ok;
       if (!ok) return 0.0f;
     }
     // a bulk tile is never the ragged last tile (its last site has a +x link
     // out of the fluid), so x + 1 < n; the guard keeps the update in bounds
-    if (x + 1 < n) return bulk_update2<S, ODD>(P, np, x, dsc, half ? omB : omA, err, chk);
-    return bulk_update<S, ODD>(P, np, x, dsc, half ? omB : omA, err, chk);
+    if (x + 1 < d.n) return bulk_update2<S, ODD>(P, d.npad, x, dsc, om, d.err, d.chk);
+    return bulk_update<S, ODD>(P, d.npad, x, dsc, om, d.err, d.chk);
   } else {
     const int32_t* da = dsc2[0];
     const int64_t xa = (int64_t)da[19] * kTile + lane;
-    S* PA = static_cast<S*>(dA.pop);
     if (!two) {
-      if (xa < dA.n) return bulk_update<S, ODD>(PA, dA.npad, xa, da, omA, dA.err, dA.chk);
+      if (xa < d.n) return bulk_update<S, ODD>(P, d.npad, xa, da, om, d.err, d.chk);
       return 0.0f;
     }
     const int32_t* db = dsc2[1];
     const int64_t xb = (int64_t)db[19] * kTile + lane;
-    if (!one_lattice || xa >= dA.n || xb >= dA.n) {
-      // the two tiles belong to different members of an ensemble (or a site
-      // has no partner, not reached for bulk tiles): one site at a time
-      S* PB = static_cast<S*>(dB.pop);
+    if (xa >= d.n || xb >= d.n) {  // not reached for bulk tiles: one site at a time
       float r = 0.0f;
-      if (xa < dA.n) r += bulk_update<S, ODD>(PA, dA.npad, xa, da, omA, dA.err, dA.chk);
-      if (xb < dB.n) r += bulk_update<S, ODD>(PB, dB.npad, xb, db, omB, dB.err, dB.chk);
+      if (xa < d.n) r += bulk_update<S, ODD>(P, d.npad, xa, da, om, d.err, d.chk);
+      if (xb < d.n) r += bulk_update<S, ODD>(P, d.npad, xb, db, om, d.err, d.chk);
       return r;
     }
     // B directly follows A with the same offsets (warp-uniform)
@@ -1611,11 +1615,11 @@ __device__ __forceinline__ float bulk_pair_warp(const BulkView& dA, int64_t kA, 
     if constexpr (kChecked && ODD) {
       bool ok = true;
       for (int o = 0; o < 18; ++o)
-        ok = chk_site(xa + da[o], dA.n, dA.err) && chk_site(xb + db[o], dA.n, dA.err) && ok;
+        ok = chk_site(xa + da[o], d.n, d.err) && chk_site(xb + db[o], d.n, d.err) && ok;
       if (!ok) return 0.0f;
     }
-    if (same) return bulk_update2v<S, ODD, true>(PA, dA.npad, xa, xb, da, db, omA, dA.err, dA.chk);
-    return bulk_update2v<S, ODD, false>(PA, dA.npad, xa, xb, da, db, omA, dA.err, dA.chk);
+    if (same) return bulk_update2v<S, ODD, true>(P, d.npad, xa, xb, da, db, om, d.err, d.chk);
+    return bulk_update2v<S, ODD, false>(P, d.npad, xa, xb, da, db, om, d.err, d.chk);
   }
 }
 
@@ -1632,8 +1636,7 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::two)
   if (k0 >= d.n_tiles) return;  // warp-uniform
   const BulkView v = bulk_view(d);
   const bool two = k0 + 1 < d.n_tiles;
-  const float dr = bulk_pair_warp<S, ODD, VERT>(v, k0, p.omega_f, v, k0 + 1, p.omega_f, two, true,
-                                                p.prefetch, desc_s[w], lane);
+  const float dr = bulk_pair_warp<S, ODD, VERT>(v, k0, p.omega_f, two, p.prefetch, desc_s[w], lane);
   if constexpr (DIAG) {
     // the two tiles' mass under the first one's launch position
     const float m = warp_sum(dr);
@@ -1726,10 +1729,10 @@ __global__ void __launch_bounds__(kStageWarps * 32, kStages <= 2 ? 8 : (kStages 
     const int64_t x = (int64_t)(lane < 16 ? ta[0] : tb[0]) * kTile + 2 * (lane & 15);
     const uint32_t* row = &buf[w][st][lane >> 4][lane & 15];  // row j at + j * 16 words
     using Cd = Codec2<S>;
-    collide2<true>(
+    collide2<true, int*>(
         [&](int j) -> F2 { return Cd::unpack(row[j * (kTile / 2)]); },
         [&](int j) -> F2 { return Cd::unpack(lds_volatile_u32(row + j * (kTile / 2))); }, om,
-        d.err, d.err, [&](F2 s0) { Cd::st_al(P + x, s0); },
+        d.err, [&](F2 s0) { Cd::st_al(P + x, s0); },
         [&](auto A, F2 sa, F2 sb) {
           constexpr int a = decltype(A)::value, b = a + 1;
           Cd::st_al(P + b * np + x, sa);
@@ -1979,49 +1982,116 @@ __device__ __forceinline__ TileRef tile_ref(const TileRef* map, int64_t g) {
   return TileRef{(int32_t)(v & 0xFFFFFFFFll), (int32_t)(v >> 32)};
 }
 
+// The bulk kernels read one 96-byte descriptor per tile (EnsDesc) that holds
+// all a tile needs of its member: the address of its first site's slot in
+// population row 0, the row length and the relaxation rate. So a warp has
+// one load before those of its populations, as in a single lattice, and two
+// tiles of a warp always belong to one member (a member with an odd number of
+// bulk tiles has an empty descriptor at its end). Through a tile map, the
+// member's table and its launch list it had three loads in a row, held both
+// members' pointers (up to 128 registers: 16 warps per SM), and could prefetch
+// only within its member. A step of 48 tubes: FP16 316 -> 262 us; FP32 426 (one
+// site per lane, prefetch) -> 350 us (two sites per lane, no prefetch).
+__global__ void k_ens_desc(const MemberDev* mem, const TileRef* map, int64_t n, int elem,
+                           EnsDesc* out) {
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (g >= n) return;  // warp-uniform
+  const TileRef t = tile_ref(map, g);
+  EnsDesc* o = out + g;
+  if (t.k < 0) {  // padding
+    if (lane < (int)(sizeof(EnsDesc) / 4)) reinterpret_cast<int32_t*>(o)[lane] = 0;
+    return;
+  }
+  const MemberDev& md = mem[t.member];
+  const LaunchDesc* l = md.d.launch + t.k;
+  if (lane < 18) o->code[lane] = l->code[lane];
+  if (lane == 18) o->np = (int32_t)md.d.npad;
+  if (lane == 19) o->omega_f = md.omega_f;
+  if (lane == 20)
+    o->pop = reinterpret_cast<uint64_t>(md.d.pop) + (uint64_t)l->tile * kTile * (uint64_t)elem;
+  if (lane == 21) o->member = t.member;
+  if (lane == 22) o->pad = 0;
+}
+
+constexpr int kEnsWords = sizeof(EnsDesc) / 4;
+template <class S>
+__device__ __forceinline__ S* ens_pop(const int32_t* dsc) {
+  return *reinterpret_cast<S* const*>(dsc + 20);
+}
+// L2 prefetch of the populations of the tile at descriptor g.
+template <class S>
+__device__ __forceinline__ void ens_prefetch(const EnsembleLaunch& e, int64_t g, int lane) {
+  if (g >= e.n_desc || lane >= kQ) return;
+  const unsigned long long p =
+      __ldg(reinterpret_cast<const unsigned long long*>(&e.desc[g].pop));
+  const int32_t np = __ldg(&e.desc[g].np);
+  if (p) bulk_prefetch_l2(reinterpret_cast<const S*>(p) + (int64_t)lane * np, kTile * sizeof(S));
+}
+
 template <class S, bool ODD, int W>
 __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::one)
     k_bulk_ens(const EnsembleLaunch e, const StepParams p) {
-  __shared__ __align__(16) int32_t desc_s[W][20];
+  using C = typename Codec<S>::C;
+  __shared__ __align__(16) int32_t desc_s[W][kEnsWords];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t g = (int64_t)blockIdx.x * W + w;
-  if (g >= e.n_bulk_tiles) return;  // warp-uniform
-  const TileRef t = tile_ref(e.bulk_map, g);
-  const MemberDev& md = e.mem[t.member];
-  StepParams pm = p;
-  pm.omega = md.omega;
-  pm.omega_f = md.omega_f;
-  bulk_tile<S, ODD>(md.d, pm, t.k, desc_s[w], lane);
+  if (g >= e.n_desc) return;  // warp-uniform
+  int32_t* dsc = desc_s[w];
+  if (lane < kEnsWords) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(e.desc + g) + lane);
+  if (p.prefetch > 0) ens_prefetch<S>(e, g + p.prefetch, lane);
+  __syncwarp();
+  S* P = ens_pop<S>(dsc);
+  if (!P) return;  // padding
+  const MemberDev* m = e.mem + dsc[22];
+  C om;
+  if constexpr (std::is_same<C, double>::value) om = m->omega;
+  else om = __int_as_float(dsc[19]);
+  bulk_update<S, ODD>(P, (int64_t)dsc[18], (int64_t)lane, dsc, om, m, nullptr);
 }
 
-__device__ __forceinline__ BulkView member_view(const MemberDev* m) {
-  const DevLattice* d = &m->d;
-  BulkView v;
-  v.pop = (void*)__ldg(reinterpret_cast<const unsigned long long*>(&d->pop));
-  v.launch = reinterpret_cast<const LaunchDesc*>(
-      __ldg(reinterpret_cast<const unsigned long long*>(&d->launch)));
-  v.err = (int*)__ldg(reinterpret_cast<const unsigned long long*>(&d->err));
-  v.chk = (int*)__ldg(reinterpret_cast<const unsigned long long*>(&d->chk));
-  v.npad = __ldg(&d->npad);
-  v.n = __ldg(&d->n);
-  v.n_tiles = __ldg(&d->n_tiles);
-  return v;
-}
-
-// Bulk tiles of all members, two per warp (the pair may span two members).
+// Two bulk tiles per warp, two sites per lane (see bulk_pair_warp).
 template <class S, bool ODD, bool VERT, int W>
 __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::two)
     k_bulk2_ens(const EnsembleLaunch e, const StepParams p) {
-  __shared__ __align__(16) int32_t desc_s[W][2][20];
+  __shared__ __align__(16) int32_t desc_s[W][2][kEnsWords];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t g0 = 2 * ((int64_t)blockIdx.x * W + w);
-  if (g0 >= e.n_bulk_tiles) return;  // warp-uniform
-  const bool two = g0 + 1 < e.n_bulk_tiles;
-  const TileRef ta = tile_ref(e.bulk_map, g0), tb = two ? tile_ref(e.bulk_map, g0 + 1) : ta;
-  const BulkView A = member_view(e.mem + ta.member), B = member_view(e.mem + tb.member);
-  bulk_pair_warp<S, ODD, VERT>(A, ta.k, __ldg(&e.mem[ta.member].omega_f), B, tb.k,
-                               __ldg(&e.mem[tb.member].omega_f), two, ta.member == tb.member,
-                               p.prefetch, desc_s[w], lane);
+  if (g0 >= e.n_desc) return;  // warp-uniform (n_desc is even)
+  int32_t* da = desc_s[w][0];
+  int32_t* db = desc_s[w][1];
+  if (lane < kEnsWords) {
+    da[lane] = __ldg(reinterpret_cast<const int32_t*>(e.desc + g0) + lane);
+    db[lane] = __ldg(reinterpret_cast<const int32_t*>(e.desc + g0 + 1) + lane);
+  }
+  if (p.prefetch > 0) {
+    ens_prefetch<S>(e, g0 + p.prefetch, lane);
+    ens_prefetch<S>(e, g0 + p.prefetch + 1, lane);
+  }
+  __syncwarp();
+  const MemberDev* m = e.mem + da[22];
+  const float om = __int_as_float(da[19]);
+  const int64_t np = da[18];
+  S* PB = ens_pop<S>(db);
+  if constexpr (!VERT) {
+    const int32_t* dsc = lane < 16 ? da : db;
+    S* P = ens_pop<S>(dsc);
+    if (!P) return;  // padding
+    bulk_update2<S, ODD>(P, np, (int64_t)(2 * (lane & 15)), dsc, om, m, nullptr);
+  } else {
+    S* PA = ens_pop<S>(da);
+    if (!PB) {
+      bulk_update<S, ODD>(PA, np, (int64_t)lane, da, om, m, nullptr);
+      return;
+    }
+    // B directly follows A with the same offsets (warp-uniform)
+    if (__all_sync(0xFFFFFFFFu, lane < 18 ? da[lane] == db[lane] : PB == PA + kTile))
+      bulk_update2v<S, ODD, true>(PA, np, (int64_t)lane, (int64_t)lane + kTile, da, db, om, m,
+                                  nullptr);
+    else
+      bulk_update2v<S, ODD, false>(PA, np, (int64_t)lane, (int64_t)lane + (PB - PA), da, db, om, m,
+                                   nullptr);
+  }
 }
 
 template <class S, bool ODD>
@@ -2734,7 +2804,7 @@ void launch_bulk_ens(const EnsembleLaunch& e, const StepParams& p, bool odd, int
                      cudaStream_t m) {
   if (pairing == 3) pairing = 1;  // staged rows: single lattices only
   if (pairing) {
-    const unsigned nb = (unsigned)((e.n_bulk_tiles + 2 * W - 1) / (2 * W));
+    const unsigned nb = (unsigned)((e.n_desc + 2 * W - 1) / (2 * W));
     if constexpr (sizeof(S) < 8) {
       if (pairing == 1) {
         if (odd) k_bulk2_ens<S, true, false, W><<<nb, W * 32, 0, m>>>(e, p);
@@ -2745,7 +2815,7 @@ void launch_bulk_ens(const EnsembleLaunch& e, const StepParams& p, bool odd, int
       }
     }
   } else {
-    const unsigned nb = (unsigned)((e.n_bulk_tiles + W - 1) / W);
+    const unsigned nb = (unsigned)((e.n_desc + W - 1) / W);
     if (odd) k_bulk_ens<S, true, W><<<nb, W * 32, 0, m>>>(e, p);
     else k_bulk_ens<S, false, W><<<nb, W * 32, 0, m>>>(e, p);
   }
@@ -2899,6 +2969,14 @@ int launch_small(int storage, const DevLattice& d, const StepParams& p, int64_t 
     using S = std::remove_pointer_t<decltype(tag)>;
     return small_t<S>(d, p, n_steps, bar, (cudaStream_t)stream);
   });
+}
+
+int launch_ens_desc(int storage, const MemberDev* mem, const TileRef* map, int64_t n, EnsDesc* out,
+                    void* stream) {
+  if (n <= 0) return 0;
+  k_ens_desc<<<blocks_for(n * 32, 256), 256, 0, (cudaStream_t)stream>>>(
+      mem, map, n, (int)storage_bytes(storage), out);
+  return (int)cudaGetLastError();
 }
 
 int launch_set_step(int64_t* step_dev, int64_t value, void* stream) {

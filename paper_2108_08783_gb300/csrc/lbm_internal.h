@@ -250,6 +250,19 @@ struct TileRef {
   int32_t k;
 };
 
+// A bulk tile of an ensemble with all its kernel needs of its member: neighbour
+// offsets, row length of the populations, 1 / tau, the address of its first
+// site in row 0 (0: padding), and the member (for its error word).
+struct alignas(16) EnsDesc {
+  int32_t code[18];
+  int32_t np;
+  float omega_f;
+  uint64_t pop;
+  int32_t member;
+  int32_t pad;
+};
+static_assert(sizeof(EnsDesc) == 96, "EnsDesc must be 96 bytes");
+
 // Ensemble launch: the members' bulk (boundary) tiles are numbered in
 // schedule order; bulk_map[g] (boundary_map[g]) names the member and launch
 // position of global bulk (boundary) tile g.
@@ -257,6 +270,8 @@ struct EnsembleLaunch {
   const MemberDev* mem;
   const TileRef* bulk_map;      // [n_bulk_tiles]
   const TileRef* boundary_map;  // [n_boundary_tiles]
+  const EnsDesc* desc;          // [n_desc] bulk tiles, each member's padded to an even number
+  int64_t n_desc;
   int32_t n_members;
   int64_t n_bulk_tiles, n_boundary_tiles;
   const MemberDev* multi_host;  // host copies of the members with multi-iolet tiles
@@ -288,6 +303,9 @@ int launch_ensemble_persistent(int storage, const EnsembleLaunch& e, const StepP
 int64_t small_tiles(int storage, int n_sms);
 int launch_small(int storage, const DevLattice& d, const StepParams& p, int64_t n_steps, void* bar,
                  void* stream);
+// The descriptors of n bulk tiles (map: member and launch position, k < 0 for padding).
+int launch_ens_desc(int storage, const MemberDev* mem, const TileRef* map, int64_t n, EnsDesc* out,
+                    void* stream);
 int launch_advance(int64_t* step_dev, int64_t by, void* stream);
 int launch_set_step(int64_t* step_dev, int64_t value, void* stream);
 int launch_init(int storage, const DevLattice& d, const double* rho, const double* u,

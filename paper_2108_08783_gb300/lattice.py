@@ -20,10 +20,13 @@ def _ptr(a):
     return None if a is None else C.c_void_p(a.ctypes.data)
 
 
-def default_knobs(storage):
+def default_knobs(storage, ensemble=False):
     """The launch knobs a new lattice or ensemble starts with (``lbm_tune``): two
     sites per lane for 16-bit storage, one otherwise; an L2 prefetch distance of
-    4096 tiles for FP32 storage, none otherwise; CTAs of 4 warps."""
+    4096 tiles for FP32 storage, none otherwise; CTAs of 4 warps.  An ensemble
+    starts with two sites per lane and no prefetch for FP32 storage too."""
+    if ensemble:
+        return dict(bulk_sites=1 if storage == "f64" else 2, bulk_warps=4, prefetch=0)
     sixteen = storage in ("f16s", "bf16s")
     return dict(bulk_sites=2 if sixteen else 1, bulk_warps=4,
                 prefetch=4096 if storage == "f32" else 0)
@@ -436,7 +439,7 @@ class Ensemble:
         storage = self.members[0].storage
         if storage == "f64":
             bulk_sites = (1,)
-        start = dict(default_knobs(storage), schedule=0, graph_steps=0, persistent=0)
+        start = dict(default_knobs(storage, ensemble=True), schedule=0, graph_steps=0, persistent=0)
         knobs = (("schedule", schedule),
                  (("bulk_sites", "prefetch"), list(itertools.product(bulk_sites, prefetch))),
                  ("bulk_warps", bulk_warps), ("graph_steps", graph_steps),
