@@ -57,6 +57,9 @@ struct lbm_ctx {
   double tau = 1.0;
   int wall_model = LBM_WALL_BOUNCEBACK;
   double rho0 = 1.0;
+  // F and kappa are the same at every wall site (zero until they are set)
+  bool wall_uniform = true;
+  double wall_F = 0.0, wall_kappa = 0.0;
   int64_t step = 0;
   cudaStream_t stream = nullptr;
   lbm_allocator alloc{};
@@ -521,6 +524,9 @@ int lbm_set_wall_params(lbm_ctx* c, int32_t wall_model, double rho0, const doubl
   if (rc != LBM_OK) return rc;
   c->wall_model = wall_model;
   c->rho0 = rho0;
+  c->wall_uniform = n == 1;
+  c->wall_F = n == 1 && F ? F[0] : 0.0;
+  c->wall_kappa = n == 1 && kappa ? kappa[0] : 0.0;
   c->gexec_steps = 0;  // a captured step graph holds the old wall constants
   return LBM_OK;
 }
@@ -585,6 +591,10 @@ lbm::StepParams step_params(const lbm_ctx* c) {
   p.omega = 1.0 / c->tau;
   p.omega_f = (float)p.omega;
   p.elastic = c->wall_model == LBM_WALL_ELASTIC_GZS ? 1 : 0;
+  p.wall_uniform = c->wall_uniform ? 1 : 0;
+  p.wall_F = c->wall_F;
+  p.wall_F_f = (float)c->wall_F;
+  p.wall_K = c->wall_kappa / 3.0;
   p.prefetch = c->prefetch;
   p.step_dev = nullptr;
   p.bulk_sites = c->bulk_sites;
@@ -1316,6 +1326,10 @@ int ens_upload(lbm_ensemble* e) {
     md.rho0_f = (float)c->rho0;
     md.rho0_exact = (double)md.rho0_f == c->rho0 ? 1 : 0;
     md.elastic = c->wall_model == LBM_WALL_ELASTIC_GZS ? 1 : 0;
+    md.wall_uniform = c->wall_uniform ? 1 : 0;
+    md.wall_F = c->wall_F;
+    md.wall_F_f = (float)c->wall_F;
+    md.wall_K = c->wall_kappa / 3.0;
   }
   cudaError_t r = cudaMemcpyAsync(e->mem_d, tab.data(), n * sizeof(lbm::MemberDev),
                                   cudaMemcpyHostToDevice, e->stream);

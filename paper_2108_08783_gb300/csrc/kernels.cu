@@ -1123,10 +1123,18 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
   // (F + dr - dx)/dr with dr = dx + dE in the compute type.
   C sw = C(0);
   if ((smask & kHasWall) && p.elastic) {
-    cp_async_wait_all();
     // F (compute type), kappa c_s^2 (FP64)
-    const C Fw = reinterpret_cast<const C*>(site)[lane];
-    const double Kw = site[kTile + lane];
+    C Fw;
+    double Kw;
+    if (p.wall_uniform) {
+      if constexpr (std::is_same<C, double>::value) Fw = p.wall_F;
+      else Fw = p.wall_F_f;
+      Kw = p.wall_K;
+    } else {
+      cp_async_wait_all();
+      Fw = reinterpret_cast<const C*>(site)[lane];
+      Kw = site[kTile + lane];
+    }
     const double dE = tube_law(Kw, m.rho, p);
     if constexpr (std::is_same<C, double>::value) {
       const double dr = 1.0 + dE;
@@ -1799,10 +1807,12 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   // per-site data and the descriptor, all in one round trip
   const bool first = !KEEP || !(kept->have & 1u);
   const uint32_t smask = first ? __ldg(d.slot_mask + slot) : kept->smask;
-  const uint32_t iom = first ? __ldg(d.slot_io + slot) : kept->iom;
   if (first && lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
   __syncwarp();
   const uint32_t tmask = (uint32_t)dsc[18];
+  // (tiles without iolet links, most of them, skip their 128 bytes)
+  uint32_t iom = 0;
+  if (tmask & kHasIolet) iom = first ? __ldg(d.slot_io + slot) : kept->iom;
   const bool irr = tmask & kIrregular;
   const int64_t x = (int64_t)dsc[19] * kTile + lane;
   // odd steps of an irregular tile: its segment table (80 words, coalesced
@@ -1836,11 +1846,15 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   // per-site wall and inlet data (F, kappa/3, inlet profile p0, ps, pc) into
   // the warp's area (from row Area::site), copied asynchronously so that no register
   // holds them while the populations load
+  // One F and kappa for the whole lattice (p.wall_uniform) come with the launch
+  // parameters instead: 384 of a boundary tile's 700 to 1,000 bytes beside its
+  // populations (2,432 in 16-bit storage, 4,864 in FP32); depth-6 tree of root
+  // radius 36: FP32 138.5 -> 137.0 us a step, FP16 106.9 -> 105.0.
   // Rows of 32 doubles: F (row 0) and p0, ps, pc (rows 2-4) in the compute
   // type at the start of their rows, kappa c_s^2 (row 1) in FP64.
   double* site = reinterpret_cast<double*>(gsm + Area::site * kTile);  // [5][32]
   auto site_row = [&](int r) { return reinterpret_cast<C*>(site + r * kTile); };
-  if (first && valid && (smask & kHasWall)) {
+  if (first && valid && (smask & kHasWall) && (PART != 0 || !p.wall_uniform)) {
     cp_async_elem(site_row(0) + lane, static_cast<const C*>(d.slot_F) + slot);
     cp_async8(site + kTile + lane, d.slot_kappa + slot);
   }
@@ -2115,6 +2129,10 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_
   pm.rho0_exact = md.rho0_exact;
   pm.diag = 0;  // ensembles: no fused diagnostics
   pm.elastic = md.elastic;
+  pm.wall_uniform = md.wall_uniform;
+  pm.wall_F_f = md.wall_F_f;
+  pm.wall_F = md.wall_F;
+  pm.wall_K = md.wall_K;
   boundary_tile<S, ODD>(md.d, pm, t.k, desc_s[w], stage[w], &bars[w], gs[w], lane);
 }
 
@@ -2224,6 +2242,7 @@ __global__ void __launch_bounds__(kPersistWarps * 32, sizeof(S) == 8 ? 1 : 4)
           pm.rho0_exact = md.rho0_exact;
           pm.diag = 0;  // ensembles: no fused diagnostics
           pm.elastic = md.elastic;
+          pm.wall_uniform = 0;
           const int64_t k = tr.k;
           const bool ok = odd ? persist_boundary<S, true>(md.d, pm, k, desc_s[w], stage[w],
                                                           &bars[w], gsm[w], lane, &phase)

@@ -312,6 +312,7 @@ int build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
       uint32_t flags = 0, nonfluid = 0;
       for (int l = 0; l < lanes; ++l) {
         flags |= site_mask[x0 + l] & (kHasWall | kHasInlet);
+        if (site_io[x0 + l] & kDirBits) flags |= kHasIolet;
         nonfluid |= site_mask[x0 + l] & kDirBits;
       }
       // coherent: in every direction, the lanes whose link is fluid share one offset

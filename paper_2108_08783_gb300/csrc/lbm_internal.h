@@ -38,6 +38,7 @@ constexpr uint32_t kIrregular = 1u << 31;  // tile: fluid-link offsets differ be
 // segment table replaces the per-site neighbour rows on odd steps.
 constexpr uint32_t kSegmented = 1u << 20;
 constexpr int kMaxSegments = 4;
+constexpr uint32_t kHasIolet = 1u << 21;  // some site of the tile has an iolet link (tile masks only)
 // Segment table of a boundary tile, in 32-bit words: [0..3] first lane of
 // each segment (32 for an unused one), then [4 + 18 q + (i - 1)] the offset
 // nbr(x, i) - x of segment q's fluid links in direction i; padded to 80.
@@ -206,6 +207,11 @@ struct StepParams {
   int32_t rho0_exact;  // rho0 == (double) rho0_f
   int32_t elastic;   // 1: elastic GZS wall, 0: bounce-back
   int32_t write_state;
+  // one F and kappa for every wall site (else from slot_F and slot_kappa)
+  int32_t wall_uniform;
+  float wall_F_f;     // (float) wall_F
+  double wall_F;
+  double wall_K;      // kappa c_s^2
   int64_t step;      // step index (plus *step_dev when step_dev is set)
   int64_t prefetch;  // L2 prefetch distance in tiles of launch order (0: off)
   const int64_t* step_dev;  // device step counter (captured graphs), or NULL
@@ -225,6 +231,10 @@ struct MemberDev {
   float omega_f;  // (float) omega
   float rho0_f;   // (float) rho0
   int32_t rho0_exact;
+  int32_t wall_uniform;
+  float wall_F_f;
+  double wall_F;
+  double wall_K;
 };
 
 
