@@ -76,6 +76,7 @@ struct lbm_ctx {
   int32_t bulk_sites = 1;  // bulk kernel mode, set from the storage at build
   int32_t bulk_warps = 4;  // warps per CTA of the bulk kernel
   int32_t n_sms = 0;       // SMs of the context's device
+  int64_t l2_bytes = 0;    // and its L2
   // captured steps (LBM_TUNE_GRAPH_STEPS): G steps replayed as one CUDA graph
   // on a private stream, ordered with the context's stream by events; the
   // inlet phase reads a device step counter that the graph advances
@@ -195,6 +196,15 @@ template <class T>
 cudaError_t h2d(lbm_ctx* c, T* dst, const T* src, size_t count) {
   if (count == 0) return cudaSuccess;
   return cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c->stream);
+}
+
+// Bytes of the populations, and whether a step should begin where the last one
+// ended (launch_step): populations beyond L2, in a storage bound by memory.
+int64_t pop_bytes(const lbm_ctx* c) {
+  return (int64_t)lbm::kQ * c->d.npad * (int64_t)lbm::storage_bytes(c->storage);
+}
+int32_t alternate(const lbm_ctx* c, int64_t bytes) {
+  return c->storage != LBM_F64 && c->l2_bytes > 0 && bytes > c->l2_bytes ? 1 : 0;
 }
 
 int check_launch(lbm_ctx* c, int rc, const char* what) {
@@ -443,10 +453,13 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
   chk(cudaMemsetAsync(err, 0, sizeof(int), c->stream));
   chk(cudaMemsetAsync(c->small_bar, 0, sizeof(unsigned long long), c->stream));
   {
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, l2 = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) == cudaSuccess) {
       c->n_sms = sms;
+      c->l2_bytes = l2;
+    }
     cudaGetLastError();
     c->small = d.n_tiles > 0 && d.n_multi == 0 && d.n_tiles <= lbm::small_tiles(storage, c->n_sms);
   }
@@ -600,6 +613,7 @@ lbm::StepParams step_params(const lbm_ctx* c) {
   p.bulk_sites = c->bulk_sites;
   p.bulk_warps = c->bulk_warps;
   p.n_sms = c->n_sms;
+  p.alternate = alternate(c, pop_bytes(c));
   p.tmap = c->tmap_ready ? &c->tmap : nullptr;
   return p;
 }
@@ -1533,6 +1547,9 @@ int lbm_ensemble_step(lbm_ensemble* e, int64_t n_steps) {
   p.prefetch = e->prefetch;
   p.bulk_sites = e->bulk_sites;
   p.bulk_warps = e->bulk_warps;
+  int64_t bytes = 0;
+  for (const lbm_ctx* c : e->members) bytes += pop_bytes(c);
+  p.alternate = alternate(e->members[0], bytes);
   int64_t done = 0;
   if (e->persistent && n_steps > 0) {
     p.step = step0;

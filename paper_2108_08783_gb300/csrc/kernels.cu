@@ -1501,6 +1501,12 @@ struct EnsBulkMinBlocks {
 #endif
 constexpr int kBoundaryWarps = LBM_BOUNDARY_WARPS;  // k_boundary: tiles (warps) per CTA
 
+// The step walks its tiles in descending order (see step_t).
+template <bool ODD>
+__device__ __forceinline__ bool descending(const StepParams& p) {
+  return ODD && p.alternate;
+}
+
 // Bulk tile at launch position k (whole warp); dsc: the warp's 20-word area.
 // Returns the lane's rho - 1 (0 for a lane without a site).  With SLOT the
 // tile's sum goes to *slot instead (fused diagnostics): from inside the update
@@ -1515,8 +1521,9 @@ __device__ __forceinline__ typename Codec<S>::C bulk_tile(const DevLattice& d,
   // with the previous tile's descriptor before it is overwritten
   __syncwarp();
   if (lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
-  if (p.prefetch > 0 && k + p.prefetch < d.n_tiles && lane < kQ) {
-    const int64_t tp = __ldg(&d.launch[k + p.prefetch].tile);
+  const int64_t kp = descending<ODD>(p) ? k - p.prefetch : k + p.prefetch;
+  if (p.prefetch > 0 && kp >= d.n_boundary && kp < d.n_tiles && lane < kQ) {
+    const int64_t tp = __ldg(&d.launch[kp].tile);
     bulk_prefetch_l2(static_cast<const S*>(d.pop) + lane * d.npad + tp * kTile,
                      kTile * sizeof(S));
   }
@@ -1571,13 +1578,16 @@ __device__ __forceinline__ BulkView bulk_view(const DevLattice& d) {
 // A site without a partner takes the single-site update.
 template <class S, bool ODD, bool VERT>
 __device__ __forceinline__ float bulk_pair_warp(const BulkView& d, int64_t k0, float om, bool two,
-                                               int64_t prefetch, int32_t (*dsc2)[20], int lane) {
+                                               const StepParams& p, int32_t (*dsc2)[20],
+                                               int lane) {
   if (lane < 20) {
     dsc2[0][lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k0) + lane);
     if (two) dsc2[1][lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k0 + 1) + lane);
   }
-  if (prefetch > 0 && lane < kQ) {
-    for (int64_t k = k0 + prefetch; k < k0 + prefetch + 2 && k < d.n_tiles; ++k) {
+  if (p.prefetch > 0 && lane < kQ) {
+    const int64_t kp = descending<ODD>(p) ? k0 - p.prefetch : k0 + p.prefetch;
+    for (int64_t k = kp; k < kp + 2 && k < d.n_tiles; ++k) {
+      if (k < 0) continue;
       const int64_t tp = __ldg(&d.launch[k].tile);
       bulk_prefetch_l2(static_cast<const S*>(d.pop) + lane * d.npad + tp * kTile,
                        kTile * sizeof(S));
@@ -1640,11 +1650,12 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::two)
     k_bulk2(const DevLattice d, const StepParams p) {
   __shared__ __align__(16) int32_t desc_s[W][2][20];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t k0 = d.n_boundary + 2 * ((int64_t)blockIdx.x * W + w);
-  if (k0 >= d.n_tiles) return;  // warp-uniform
+  const int64_t q = (int64_t)blockIdx.x * W + w, pairs = (d.n_tiles - d.n_boundary + 1) / 2;
+  if (q >= pairs) return;  // warp-uniform
+  const int64_t k0 = d.n_boundary + 2 * (descending<ODD>(p) ? pairs - 1 - q : q);
   const BulkView v = bulk_view(d);
   const bool two = k0 + 1 < d.n_tiles;
-  const float dr = bulk_pair_warp<S, ODD, VERT>(v, k0, p.omega_f, two, p.prefetch, desc_s[w], lane);
+  const float dr = bulk_pair_warp<S, ODD, VERT>(v, k0, p.omega_f, two, p, desc_s[w], lane);
   if constexpr (DIAG) {
     // the two tiles' mass under the first one's launch position
     const float m = warp_sum(dr);
@@ -1764,8 +1775,9 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::one)
     k_bulk(const DevLattice d, const StepParams p) {
   __shared__ __align__(16) int32_t desc_s[W][20];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t k = d.n_boundary + (int64_t)blockIdx.x * W + w;
-  if (k >= d.n_tiles) return;  // warp-uniform
+  const int64_t q = (int64_t)blockIdx.x * W + w;
+  if (q >= d.n_tiles - d.n_boundary) return;  // warp-uniform
+  const int64_t k = descending<ODD>(p) ? d.n_tiles - 1 - q : d.n_boundary + q;
   if constexpr (DIAG) bulk_tile<S, ODD, true>(d, p, k, desc_s[w], lane, d.diag_mass + k);
   else bulk_tile<S, ODD>(d, p, k, desc_s[w], lane);
 }
@@ -1950,8 +1962,9 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_
   __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t k = (int64_t)blockIdx.x * kBoundaryWarps + w;
-  if (k >= d.n_boundary) return;  // warp-uniform
+  const int64_t q = (int64_t)blockIdx.x * kBoundaryWarps + w;
+  if (q >= d.n_boundary) return;  // warp-uniform
+  const int64_t k = descending<ODD>(p) ? d.n_boundary - 1 - q : q;
   C dr = C(0);
   boundary_tile<S, ODD>(d, p, k, desc_s[w], stage[w], &bars[w], gs[w], lane, nullptr, &dr);
   if constexpr (DIAG) {
@@ -2036,7 +2049,7 @@ __device__ __forceinline__ S* ens_pop(const int32_t* dsc) {
 // L2 prefetch of the populations of the tile at descriptor g.
 template <class S>
 __device__ __forceinline__ void ens_prefetch(const EnsembleLaunch& e, int64_t g, int lane) {
-  if (g >= e.n_desc || lane >= kQ) return;
+  if (g < 0 || g >= e.n_desc || lane >= kQ) return;
   const unsigned long long p =
       __ldg(reinterpret_cast<const unsigned long long*>(&e.desc[g].pop));
   const int32_t np = __ldg(&e.desc[g].np);
@@ -2049,11 +2062,12 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::one)
   using C = typename Codec<S>::C;
   __shared__ __align__(16) int32_t desc_s[W][kEnsWords];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t g = (int64_t)blockIdx.x * W + w;
-  if (g >= e.n_desc) return;  // warp-uniform
+  const int64_t q = (int64_t)blockIdx.x * W + w;
+  if (q >= e.n_desc) return;  // warp-uniform
+  const int64_t g = descending<ODD>(p) ? e.n_desc - 1 - q : q;
   int32_t* dsc = desc_s[w];
   if (lane < kEnsWords) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(e.desc + g) + lane);
-  if (p.prefetch > 0) ens_prefetch<S>(e, g + p.prefetch, lane);
+  if (p.prefetch > 0) ens_prefetch<S>(e, descending<ODD>(p) ? g - p.prefetch : g + p.prefetch, lane);
   __syncwarp();
   S* P = ens_pop<S>(dsc);
   if (!P) return;  // padding
@@ -2070,8 +2084,9 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::two)
     k_bulk2_ens(const EnsembleLaunch e, const StepParams p) {
   __shared__ __align__(16) int32_t desc_s[W][2][kEnsWords];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t g0 = 2 * ((int64_t)blockIdx.x * W + w);
-  if (g0 >= e.n_desc) return;  // warp-uniform (n_desc is even)
+  const int64_t q = 2 * ((int64_t)blockIdx.x * W + w);
+  if (q >= e.n_desc) return;  // warp-uniform (n_desc is even)
+  const int64_t g0 = descending<ODD>(p) ? e.n_desc - 2 - q : q;
   int32_t* da = desc_s[w][0];
   int32_t* db = desc_s[w][1];
   if (lane < kEnsWords) {
@@ -2079,8 +2094,9 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::two)
     db[lane] = __ldg(reinterpret_cast<const int32_t*>(e.desc + g0 + 1) + lane);
   }
   if (p.prefetch > 0) {
-    ens_prefetch<S>(e, g0 + p.prefetch, lane);
-    ens_prefetch<S>(e, g0 + p.prefetch + 1, lane);
+    const int64_t gp = descending<ODD>(p) ? g0 - p.prefetch : g0 + p.prefetch;
+    ens_prefetch<S>(e, gp, lane);
+    ens_prefetch<S>(e, gp + 1, lane);
   }
   __syncwarp();
   const MemberDev* m = e.mem + da[22];
@@ -2117,8 +2133,9 @@ __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_
   __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t g = (int64_t)blockIdx.x * kBoundaryWarps + w;
-  if (g >= e.n_boundary_tiles) return;  // warp-uniform
+  const int64_t q = (int64_t)blockIdx.x * kBoundaryWarps + w;
+  if (q >= e.n_boundary_tiles) return;  // warp-uniform
+  const int64_t g = descending<ODD>(p) ? e.n_boundary_tiles - 1 - q : q;
   const TileRef t = tile_ref(e.boundary_map, g);
   const MemberDev& md = e.mem[t.member];
   StepParams pm = p;
@@ -2840,41 +2857,83 @@ void launch_bulk_ens(const EnsembleLaunch& e, const StepParams& p, bool odd, int
   }
 }
 
-// One step: k_boundary on the side stream, k_bulk on the main stream, joined
-// on the main stream.  ev (profiling): before the fork, after k_bulk, after
-// the join, all on the main stream.
+// One step, its two kernels on two streams, joined on the main one. The kernel on
+// the higher-priority side stream is dispatched first and the other fills in
+// behind it: k_boundary before k_bulk on even steps, k_bulk before k_boundary on
+// odd ones, which also walk their tiles in descending order. So a step begins
+// with the tiles the step before it ended with, and what they wrote is read
+// from L2 (129 MB, of the long tube's 196 MB in 16-bit storage and 391 MB in
+// FP32) instead of DRAM: tube FP16 86.9 -> 80.9 us a step, FP32 127.1 -> 122.9;
+// depth-6 tree of root radius 36 (164 and 329 MB) FP16 105.0 -> 99.7, FP32
+// 137.0 -> 131.1; 48 tubes (471 and 943 MB) FP16 261.8 -> 251.6, FP32 351 -> 343; descending odd steps alone, with k_boundary always first, gave
+// 82.9, 126.0, 103.5 and 135.9. Populations that fit L2 stay there in any order,
+// and FP64 steps are bound by the FP64 pipe: both keep k_boundary, whose tiles
+// take longest, first and ascending order (p.alternate = 0; 162,000 sites in
+// FP32: 5.5 us a step, 5.7 with odd steps descending, 7.0 with the kernels
+// changing places too).
+// ev (profiling): before the fork, after k_bulk, after the join, all on the main
+// stream, which then always has k_bulk.
+struct StepOrder {
+  cudaStream_t boundary, bulk;
+  bool fork, bulk_first;
+};
+inline StepOrder step_order(const StepStreams& ss, bool odd, bool any_boundary, bool any_bulk,
+                            bool alternate) {
+  cudaStream_t m = (cudaStream_t)ss.main, side = (cudaStream_t)ss.side;
+  StepOrder o{m, m, any_boundary && any_bulk, odd && alternate};
+  if (o.fork) (o.bulk_first ? o.bulk : o.boundary) = side;
+  return o;
+}
+inline void step_fork(const StepStreams& ss, const StepOrder& o) {
+  if (!o.fork) return;
+  cudaEventRecord((cudaEvent_t)ss.fork, (cudaStream_t)ss.main);
+  cudaStreamWaitEvent((cudaStream_t)ss.side, (cudaEvent_t)ss.fork, 0);
+}
+inline void step_join(const StepStreams& ss, const StepOrder& o) {
+  if (!o.fork) return;
+  cudaEventRecord((cudaEvent_t)ss.join, (cudaStream_t)ss.side);
+  cudaStreamWaitEvent((cudaStream_t)ss.main, (cudaEvent_t)ss.join, 0);
+}
+
 template <class S>
 int step_t(const DevLattice& d, const StepParams& p, const StepStreams& ss, void* const* ev) {
-  cudaStream_t m = (cudaStream_t)ss.main, side = (cudaStream_t)ss.side;
-
+  cudaStream_t m = (cudaStream_t)ss.main;
   const unsigned nbnd = (unsigned)((d.n_boundary + kBoundaryWarps - 1) / kBoundaryWarps);
   const int64_t nbulk_tiles = d.n_tiles - d.n_boundary;
   const bool odd = p.step & 1;
-  if (ev) cudaEventRecord((cudaEvent_t)ev[0], m);
-  if (nbnd) {
-    cudaEventRecord((cudaEvent_t)ss.fork, m);
-    cudaStreamWaitEvent(side, (cudaEvent_t)ss.fork, 0);
+  const StepOrder o = step_order(ss, odd, nbnd > 0, nbulk_tiles > 0,
+                                 p.alternate && !ev);
+  auto boundary = [&]() {
+    if (!nbnd) return;
+    cudaStream_t s = o.boundary;
     if (p.diag) {
-      if (odd) k_boundary<S, true, true><<<nbnd, kBoundaryWarps * 32, 0, side>>>(d, p);
-      else k_boundary<S, false, true><<<nbnd, kBoundaryWarps * 32, 0, side>>>(d, p);
+      if (odd) k_boundary<S, true, true><<<nbnd, kBoundaryWarps * 32, 0, s>>>(d, p);
+      else k_boundary<S, false, true><<<nbnd, kBoundaryWarps * 32, 0, s>>>(d, p);
     } else {
-      if (odd) k_boundary<S, true><<<nbnd, kBoundaryWarps * 32, 0, side>>>(d, p);
-      else k_boundary<S, false><<<nbnd, kBoundaryWarps * 32, 0, side>>>(d, p);
+      if (odd) k_boundary<S, true><<<nbnd, kBoundaryWarps * 32, 0, s>>>(d, p);
+      else k_boundary<S, false><<<nbnd, kBoundaryWarps * 32, 0, s>>>(d, p);
     }
-    launch_multi<S>(d, p, odd, side);
-  }
-  if (nbulk_tiles > 0) {
+    launch_multi<S>(d, p, odd, s);
+  };
+  auto bulk = [&]() {
+    if (nbulk_tiles <= 0) return;
     const int pairing = sizeof(S) < 8 ? bulk_pairing(p.bulk_sites, odd) : 0;
     // diagnostic steps take CTAs of 4 warps whatever the knob (same results)
-    if (p.diag) launch_bulk<S, 4, true>(d, p, odd, pairing, nbulk_tiles, m);
-    else if (p.bulk_warps == 8) launch_bulk<S, 8>(d, p, odd, pairing, nbulk_tiles, m);
-    else launch_bulk<S, 4>(d, p, odd, pairing, nbulk_tiles, m);
+    if (p.diag) launch_bulk<S, 4, true>(d, p, odd, pairing, nbulk_tiles, o.bulk);
+    else if (p.bulk_warps == 8) launch_bulk<S, 8>(d, p, odd, pairing, nbulk_tiles, o.bulk);
+    else launch_bulk<S, 4>(d, p, odd, pairing, nbulk_tiles, o.bulk);
+  };
+  if (ev) cudaEventRecord((cudaEvent_t)ev[0], m);
+  step_fork(ss, o);
+  if (o.bulk_first) {
+    bulk();
+    boundary();
+  } else {
+    boundary();
+    bulk();
   }
   if (ev) cudaEventRecord((cudaEvent_t)ev[1], m);
-  if (nbnd) {
-    cudaEventRecord((cudaEvent_t)ss.join, side);
-    cudaStreamWaitEvent(m, (cudaEvent_t)ss.join, 0);
-  }
+  step_join(ss, o);
   if (ev) cudaEventRecord((cudaEvent_t)ev[2], m);
   return (int)cudaGetLastError();
 }
@@ -2914,14 +2973,14 @@ int launch_step(int storage, const DevLattice& d, const StepParams& p, const Ste
 
 template <class S>
 int ensemble_step_t(const EnsembleLaunch& e, const StepParams& p, const StepStreams& ss) {
-  cudaStream_t m = (cudaStream_t)ss.main, side = (cudaStream_t)ss.side;
   const unsigned nbnd = (unsigned)((e.n_boundary_tiles + kBoundaryWarps - 1) / kBoundaryWarps);
   const bool odd = p.step & 1;  // every member is at the same step; graphs keep the parity
-  if (nbnd) {
-    cudaEventRecord((cudaEvent_t)ss.fork, m);
-    cudaStreamWaitEvent(side, (cudaEvent_t)ss.fork, 0);
-    if (odd) k_boundary_ens<S, true><<<nbnd, kBoundaryWarps * 32, 0, side>>>(e, p);
-    else k_boundary_ens<S, false><<<nbnd, kBoundaryWarps * 32, 0, side>>>(e, p);
+  const StepOrder o = step_order(ss, odd, nbnd > 0, e.n_desc > 0, p.alternate);
+  auto boundary = [&]() {
+    if (!nbnd) return;
+    cudaStream_t s = o.boundary;
+    if (odd) k_boundary_ens<S, true><<<nbnd, kBoundaryWarps * 32, 0, s>>>(e, p);
+    else k_boundary_ens<S, false><<<nbnd, kBoundaryWarps * 32, 0, s>>>(e, p);
     for (int32_t q = 0; q < e.n_multi_members; ++q) {
       const MemberDev& md = e.multi_host[q];
       StepParams pm = p;
@@ -2932,18 +2991,24 @@ int ensemble_step_t(const EnsembleLaunch& e, const StepParams& p, const StepStre
       pm.rho0_exact = md.rho0_exact;
       pm.diag = 0;  // ensembles: no fused diagnostics
       pm.elastic = md.elastic;
-      launch_multi<S>(md.d, pm, odd, side);
+      launch_multi<S>(md.d, pm, odd, s);
     }
-  }
-  if (e.n_bulk_tiles > 0) {
+  };
+  auto bulk = [&]() {
+    if (e.n_desc <= 0) return;
     const int pairing = sizeof(S) < 8 ? bulk_pairing(p.bulk_sites, odd) : 0;
-    if (p.bulk_warps == 8) launch_bulk_ens<S, 8>(e, p, odd, pairing, m);
-    else launch_bulk_ens<S, 4>(e, p, odd, pairing, m);
+    if (p.bulk_warps == 8) launch_bulk_ens<S, 8>(e, p, odd, pairing, o.bulk);
+    else launch_bulk_ens<S, 4>(e, p, odd, pairing, o.bulk);
+  };
+  step_fork(ss, o);
+  if (o.bulk_first) {
+    bulk();
+    boundary();
+  } else {
+    boundary();
+    bulk();
   }
-  if (nbnd) {
-    cudaEventRecord((cudaEvent_t)ss.join, side);
-    cudaStreamWaitEvent(m, (cudaEvent_t)ss.join, 0);
-  }
+  step_join(ss, o);
   return (int)cudaGetLastError();
 }
 

@@ -219,6 +219,7 @@ struct StepParams {
   int32_t bulk_warps;       // warps per CTA of the bulk kernel: 4 or 8
   int32_t diag;             // 1: the step kernels also write the fused diagnostics
   int32_t n_sms;            // SMs of the device (fixed-grid kernels)
+  int32_t alternate;        // 1: the two kernels change places on odd steps
   const void* tmap;         // host CUtensorMap of the populations (staged rows), or NULL
 };
 
