@@ -83,9 +83,10 @@ struct lbm_ctx {
   int64_t graph_steps = 0;
   cudaStream_t gstream = nullptr;
   cudaEvent_t g_in = nullptr, g_out = nullptr;
-  cudaGraphExec_t gexec = nullptr;
-  int gexec_parity = -1;
-  int64_t gexec_steps = 0;
+  // one graph for each parity of the first step, so that calls of an odd number
+  // of steps do not capture again each time (a fifth of a millisecond)
+  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  int64_t gexec_steps[2] = {0, 0};  // 0: capture (again) before use
   // device step counter: holds the even floor of the step it was last made
   // right for (step_d_for; -1: unknown); the captured kernels add it to their
   // compile-time offset (the parity plus the step within the block)
@@ -247,7 +248,8 @@ void lbm_destroy(lbm_ctx* c) {
   if (c->side) cudaStreamSynchronize(c->side);
   if (c->diag_stream) cudaStreamSynchronize(c->diag_stream);
   if (c->gstream) cudaStreamSynchronize(c->gstream);
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  for (cudaGraphExec_t g : c->gexec)
+    if (g) cudaGraphExecDestroy(g);
   if (c->g_in) cudaEventDestroy(c->g_in);
   if (c->g_out) cudaEventDestroy(c->g_out);
   if (c->gstream) cudaStreamDestroy(c->gstream);
@@ -540,7 +542,7 @@ int lbm_set_wall_params(lbm_ctx* c, int32_t wall_model, double rho0, const doubl
   c->wall_uniform = n == 1;
   c->wall_F = n == 1 && F ? F[0] : 0.0;
   c->wall_kappa = n == 1 && kappa ? kappa[0] : 0.0;
-  c->gexec_steps = 0;  // a captured step graph holds the old wall constants
+  c->gexec_steps[0] = c->gexec_steps[1] = 0;  // captured steps hold the old wall constants
   return LBM_OK;
 }
 
@@ -588,11 +590,10 @@ int make_tmap(lbm_ctx* c) {
 
 // n_steps timesteps; with diag_last the last one also writes the fused
 // diagnostics of the state it reads.
-void drop_graph(lbm_ctx* c) {
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  c->gexec = nullptr;
-  c->gexec_parity = -1;
-  c->gexec_steps = 0;
+void drop_graph(lbm_ctx* c, int parity) {
+  if (c->gexec[parity]) cudaGraphExecDestroy(c->gexec[parity]);
+  c->gexec[parity] = nullptr;
+  c->gexec_steps[parity] = 0;
 }
 
 // The launch parameters of the context's steps (the step index set per step).
@@ -660,8 +661,8 @@ int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
     if (r != cudaSuccess) return cuda_fail(c, r, "graph ordering");
     const lbm::StepStreams gs{c->gstream, c->side, c->fork, c->join};
     const int parity = (int)(c->step & 1);
-    if (!c->gexec || c->gexec_parity != parity || c->gexec_steps != G) {
-      drop_graph(c);
+    if (!c->gexec[parity] || c->gexec_steps[parity] != G) {
+      drop_graph(c, parity);
       cudaGraph_t graph = nullptr;
       r = cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeThreadLocal);
       for (int64_t s = 0; s < G && r == cudaSuccess; ++s) {
@@ -674,19 +675,19 @@ int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
       if (r == cudaSuccess) r = (cudaError_t)lbm::launch_advance(c->step_d, G, c->gstream);
       cudaError_t r2 = cudaStreamEndCapture(c->gstream, &graph);
       if (r == cudaSuccess) r = r2;
-      if (r == cudaSuccess) r = cudaGraphInstantiate(&c->gexec, graph, 0);
+      if (r == cudaSuccess) r = cudaGraphInstantiate(&c->gexec[parity], graph, 0);
       if (graph) cudaGraphDestroy(graph);
       if (r != cudaSuccess) {
-        c->gexec = nullptr;
+        c->gexec[parity] = nullptr;
         return cuda_fail(c, r, "step graph capture");
       }
-      c->gexec_parity = parity;
-      c->gexec_steps = G;
+      c->gexec_steps[parity] = G;
     }
     if (c->step_d_for != c->step)
       r = (cudaError_t)lbm::launch_set_step(c->step_d, c->step - parity, c->gstream);
     int64_t done = 0;
-    for (; r == cudaSuccess && n_steps - done >= G; done += G) r = cudaGraphLaunch(c->gexec, c->gstream);
+    for (; r == cudaSuccess && n_steps - done >= G; done += G)
+      r = cudaGraphLaunch(c->gexec[parity], c->gstream);
     if (r != cudaSuccess) return cuda_fail(c, r, "step graph launch");
     c->step += done;
     c->step_d_for = c->step;  // each replay advanced the counter by G
@@ -863,7 +864,7 @@ int lbm_step_diag(lbm_ctx* c, int64_t n_steps, double* out) {
 int lbm_tune(lbm_ctx* c, int32_t knob, int64_t value) {
   if (!c) return LBM_EINVAL;
   c->err.clear();
-  c->gexec_steps = 0;  // a captured step graph holds the old settings: capture again
+  c->gexec_steps[0] = c->gexec_steps[1] = 0;  // captured steps hold the old settings
   c->tuned = true;     // the launches asked for, whatever the size
   switch (knob) {
     case LBM_TUNE_GRAPH_STEPS:
