@@ -414,6 +414,7 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
     t.u_amp = s.u_amp;
     t.period = s.period > 0.0 ? s.period : 1.0;
     t.phase = s.phase;
+    t.finite = s.phase - s.phase;
     const double an = std::sqrt(s.axis[0] * s.axis[0] + s.axis[1] * s.axis[1] + s.axis[2] * s.axis[2]);
     for (int a = 0; a < 3; ++a) t.axis[a] = s.axis[a] / an;
     // fixed-point phase (fraction of a period, units of 2^-64)

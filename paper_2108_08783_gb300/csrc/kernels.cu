@@ -212,17 +212,20 @@ __device__ __forceinline__ float omega_as<float>(double, float wf) { return wf; 
 
 // Velocity inlet (Sec. 3) of a site with profile values (p0, ps, pc) at step
 // n: u_in = axis (u_mean p0 + u_amp (ps sin th + pc cos th)),
-// th = 2 pi n / T + phase.  FP64 paths take sin/cos of th in FP64, as the
-// oracle does.  FP32 paths take th from the iolet's 64-bit fixed-point phase
-// (frac(n / T + phase / 2 pi) in integer arithmetic, exact modulo one
-// period), keep its top 24 bits (a phase error below 2^-24 of a period,
-// ~4e-7 rad) and evaluate sinpi/cospi and the profile in FP32.
+// th = 2 pi n / T + phase, from the iolet's 64-bit fixed-point phase
+// (frac(n / T + phase / 2 pi) in integer arithmetic, exact modulo one period).
+// FP64 paths keep its top 53 bits (7e-16 rad, as exact as 2 pi n / T + phase
+// rounded to FP64, which loses more the larger n is) and take sinpi and cospi in
+// FP64: no range reduction, which with sin and cos of th was a third of the FP64
+// operations of an inlet tile.  FP32 paths keep 24 bits (a phase error below
+// 2^-24 of a period, ~4e-7 rad) and evaluate sinpi/cospi and the profile in FP32.
 __device__ __forceinline__ void inlet_velocity(const IoletDev& io, int64_t n, double p0, double ps,
                                                double pc, double& ux, double& uy, double& uz) {
   double g = mul_pin(io.u_mean, p0);
   if (!io.steady) {
     double sn, cs;
-    sincos(2.0 * M_PI * (double)n / io.period + io.phase, &sn, &cs);
+    const uint64_t ph = io.phase_off + (uint64_t)n * io.phase_inc;  // mod 2^64
+    sincospi(__fma_rn((double)(ph >> 11), 0x1p-52, io.finite), &sn, &cs);
     g = fma_pin(io.u_amp, fma_pin(ps, sn, mul_pin(pc, cs)), g);
   }
   ux = mul_pin(g, io.axis[0]);
@@ -1137,8 +1140,13 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
     }
     const double dE = tube_law(Kw, m.rho, p);
     if constexpr (std::is_same<C, double>::value) {
-      const double dr = 1.0 + dE;
-      sw = (Fw + dr - 1.0) / dr;
+      // dr >= 1: 1/dr from the estimate (2^-40), one Newton step, and one on the
+      // quotient's residual, in place of a general division
+      const double dr = 1.0 + dE, num = Fw + dE;
+      double y = rcp_estimate(dr);
+      y = __fma_rn(y, __fma_rn(-dr, y, 1.0), y);
+      const double q = __dmul_rn(num, y);
+      sw = __fma_rn(__fma_rn(-dr, q, num), y, q);
     } else {
       const float e = (float)dE;
       sw = (Fw + e) * recip(1.0f + e);

@@ -82,7 +82,7 @@ struct IoletDev {
   double rho;
   double u_mean, u_amp, period, phase;
   double axis[3];  // unit vector
-  double pad;
+  double finite;   // 0, or NaN when the phase is not finite
   // The same constants for the FP32 compute paths, rounded once on the host:
   // the phase th = 2 pi n / T + phase as a 64-bit fixed-point fraction of a
   // period, frac(n / T + phase / 2 pi) = (phase_off + n phase_inc) / 2^64
