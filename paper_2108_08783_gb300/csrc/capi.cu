@@ -1267,6 +1267,7 @@ struct lbm_ensemble {
   lbm::TileRef* map_d = nullptr;  // tile maps: bulk tiles, then boundary tiles
   lbm::EnsDesc* desc_d = nullptr;  // bulk tile descriptors, members padded to even numbers
   int64_t n_desc = 0;
+  lbm::EnsBoundaryDesc* bdesc_d = nullptr;  // boundary tile descriptors
   int64_t n_bulk = 0, n_boundary = 0;  // tiles of all members
   int64_t* step_d = nullptr;      // device step counter of captured graphs
   std::vector<int32_t> order;     // schedule: member order in the launch numbering
@@ -1359,6 +1360,13 @@ int ens_upload(lbm_ensemble* e) {
   e->launch.mem = e->mem_d;
   e->launch.n_members = n;
   e->launch.desc = e->desc_d;
+  e->launch.bdesc = e->bdesc_d;
+  e->launch.elastic_all = tab[0].elastic;
+  e->launch.uniform_all = 1;
+  for (const lbm::MemberDev& md : tab) {
+    if (md.elastic != tab[0].elastic) e->launch.elastic_all = -1;
+    if (!md.wall_uniform) e->launch.uniform_all = 0;
+  }
   e->launch.n_desc = e->n_desc;
   e->launch.n_bulk_tiles = e->n_bulk;
   e->launch.n_boundary_tiles = e->n_boundary;
@@ -1366,10 +1374,16 @@ int ens_upload(lbm_ensemble* e) {
   return LBM_OK;
 }
 
-// The bulk tiles' descriptors in schedule order, from the members' launch lists
-// (after ens_upload: the kernel reads the member table).
+// The tiles' descriptors in schedule order, from the members' launch lists
+// (after ens_maps and ens_upload: the kernels read the tile map and the member table).
 int ens_descs(lbm_ensemble* e) {
-  if (e->n_desc == 0) return LBM_OK;
+  cudaError_t rb = (cudaError_t)lbm::launch_ens_bdesc(e->mem_d, e->launch.boundary_map,
+                                                      e->n_boundary, e->bdesc_d, e->stream);
+  if (rb != cudaSuccess) return ens_cuda(e, rb, "ensemble descriptors");
+  if (e->n_desc == 0) {
+    rb = cudaStreamSynchronize(e->stream);
+    return rb == cudaSuccess ? LBM_OK : ens_cuda(e, rb, "ensemble descriptors");
+  }
   std::vector<lbm::TileRef> map;
   map.reserve((size_t)e->n_desc);
   for (int q = 0; q < (int)e->members.size(); ++q) {
@@ -1462,9 +1476,11 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
       alloc(std::max<int64_t>(1, e->n_bulk + e->n_boundary) * sizeof(lbm::TileRef)));
   e->desc_d = static_cast<lbm::EnsDesc*>(
       alloc(std::max<int64_t>(1, e->n_desc) * sizeof(lbm::EnsDesc)));
+  e->bdesc_d = static_cast<lbm::EnsBoundaryDesc*>(
+      alloc(std::max<int64_t>(1, e->n_boundary) * sizeof(lbm::EnsBoundaryDesc)));
   e->step_d = static_cast<int64_t*>(alloc(sizeof(int64_t)));
   e->sync_d = static_cast<lbm::GridSync*>(alloc(sizeof(lbm::GridSync)));
-  if (!e->mem_d || !e->map_d || !e->desc_d || !e->step_d || !e->sync_d) {
+  if (!e->mem_d || !e->map_d || !e->desc_d || !e->bdesc_d || !e->step_d || !e->sync_d) {
     lbm_ensemble_destroy(e);
     return LBM_ENOMEM;
   }

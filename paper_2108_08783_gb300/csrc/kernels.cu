@@ -1054,8 +1054,8 @@ constexpr bool opposites_adjacent() {
 }
 static_assert(opposites_adjacent(), "opposite directions must be adjacent");
 
-template <class S, bool ODD, class AREA>
-__device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& d,
+template <class S, bool ODD, class AREA, class D>
+__device__ __forceinline__ typename Codec<S>::C boundary_fast(const D& d,
                                                               const StepParams& p,
                                               typename Codec<S>::C omega, S* P, int64_t x,
                                               const int32_t* offp, int ostride, uint32_t smask,
@@ -1253,7 +1253,8 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const DevLattice& 
     chk_count(d.chk, P, pa, kQ * np, d.err);
     chk_count(d.chk, P, pb, kQ * np, d.err);
   });
-  if (p.diag && (iom & kDirBits)) diag_momentum(d, slot, m);
+  if constexpr (std::is_same<D, DevLattice>::value)  // ensembles have no fused diagnostics
+    if (p.diag && (iom & kDirBits)) diag_momentum(d, slot, m);
   return m.drho;
 }
 
@@ -1810,13 +1811,15 @@ struct KeptTile {
   uint32_t have;  // bit 0: loaded; bit 1: the odd steps' neighbour tables too
   uint32_t smask, iom;
 };
-template <class S, bool ODD, int PART = 0, bool KEEP = false>
-__device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepParams& p, int64_t k,
+// LOADED: the descriptor is in dsc and the lane's mask is loaded_mask (ensembles).
+template <class S, bool ODD, int PART = 0, bool KEEP = false, bool LOADED = false, class D>
+__device__ __forceinline__ bool boundary_tile(const D& d, const StepParams& p, int64_t k,
                                               int32_t* dsc, int32_t* nbr_s, uint64_t* bar,
                                               typename Codec<S>::C* gsm, int lane,
                                               uint32_t* bar_phase = nullptr,
                                               typename Codec<S>::C* dr = nullptr,
-                                              KeptTile* kept = nullptr) {
+                                              KeptTile* kept = nullptr,
+                                              uint32_t loaded_mask = 0) {
   using C = typename Codec<S>::C;
   using Area = TileArea<C, PART>;
   // a warp that updates tiles in a loop (persistent kernel): lanes that left
@@ -1826,8 +1829,11 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   const int64_t slot = k * kTile + lane;  // boundary tiles lead the launch order
   // per-site data and the descriptor, all in one round trip
   const bool first = !KEEP || !(kept->have & 1u);
-  const uint32_t smask = first ? __ldg(d.slot_mask + slot) : kept->smask;
-  if (first && lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
+  uint32_t smask = loaded_mask;
+  if constexpr (!LOADED) {
+    smask = first ? __ldg(d.slot_mask + slot) : kept->smask;
+    if (first && lane < 20) dsc[lane] = __ldg(reinterpret_cast<const int32_t*>(d.launch + k) + lane);
+  }
   __syncwarp();
   const uint32_t tmask = (uint32_t)dsc[18];
   // (tiles without iolet links, most of them, skip their 128 bytes)
@@ -1940,7 +1946,7 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
     }
     return true;
   }
-  if constexpr (PART == 0) return true;
+  if constexpr (PART != 0) {
   cp_async_wait_all();
   const C Fw = site_row(0)[lane];
   const double Kw = site[kTile + lane];
@@ -1955,6 +1961,7 @@ __device__ __forceinline__ bool boundary_tile(const DevLattice& d, const StepPar
   } else {
     boundary_slow<S, ODD>(d, p, P, x, dsc, irr, smask, iom, Fw, Kw, pr0, pr1, pr2, nbr_s, lane,
                           slot, gsm);
+  }
   }
   return true;
 }
@@ -2132,33 +2139,90 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::two)
   }
 }
 
+// The boundary kernels likewise read one 256-byte descriptor per tile. A tile
+// map, the member's table, its launch list and masks were four dependent loads
+// before the first population (44 % of the issue slots used on even steps, the
+// rest waiting for memory; a single lattice's boundary kernel, with two, 62 %).
+// A step of 48 tubes, 92,000 boundary tiles: FP16 266 -> 256 us, FP32 357 -> 347.
+__global__ void k_ens_bdesc(const MemberDev* mem, const TileRef* map, int64_t n,
+                            EnsBoundaryDesc* out) {
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (g >= n) return;  // warp-uniform
+  const TileRef t = tile_ref(map, g);
+  const MemberDev& md = mem[t.member];
+  EnsBoundaryDesc* o = out + g;
+  if (lane < 20)
+    reinterpret_cast<int32_t*>(&o->launch)[lane] =
+        __ldg(reinterpret_cast<const int32_t*>(md.d.launch + t.k) + lane);
+  if (lane == 20) o->pop = reinterpret_cast<uint64_t>(md.d.pop);
+  if (lane == 21) o->np = (int32_t)md.d.npad;
+  if (lane == 22) o->member = t.member;
+  if (lane == 23) o->slot_io = reinterpret_cast<uint64_t>(md.d.slot_io);
+  if (lane == 24) o->seg_tab = reinterpret_cast<uint64_t>(md.d.seg_tab);
+  if (lane == 25) o->k = t.k;
+  if (lane == 26) o->omega_f = md.omega_f;
+  if (lane == 27) o->pad[0] = o->pad[1] = 0;
+  o->mask[lane] = __ldg(md.d.slot_mask + (int64_t)t.k * kTile + lane);
+}
+
+// A member's lattice as boundary_tile sees it: what the descriptor holds, and
+// the rest as references into the member table, read where they are used.
+struct EnsView {
+  void* pop;
+  int64_t npad;
+  const uint32_t* slot_io;
+  const int32_t* seg_tab;
+  const int64_t& n;
+  const int32_t* const& slot_nbr;
+  const void* const& slot_prof;
+  const void* const& slot_F;
+  const double* const& slot_kappa;
+  double* const& slot_dE;
+  double* const& slot_Uw;
+  const int64_t& slot_stride;
+  const IoletDev* const& iolets;
+  int* const& err;
+  int* const& chk;
+};
+
 template <class S, bool ODD>
 __global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_ENS_BOUNDARY_MINB)
     k_boundary_ens(const EnsembleLaunch e, const StepParams p) {
   using C = typename Codec<S>::C;
   __shared__ __align__(128) int32_t stage[kBoundaryWarps][18 * kTile];
   __shared__ __align__(16) C gs[kBoundaryWarps][TileArea<C, 0>::size];
-  __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][20];
+  __shared__ __align__(16) int32_t desc_s[kBoundaryWarps][32];
   __shared__ uint64_t bars[kBoundaryWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t q = (int64_t)blockIdx.x * kBoundaryWarps + w;
   if (q >= e.n_boundary_tiles) return;  // warp-uniform
   const int64_t g = descending<ODD>(p) ? e.n_boundary_tiles - 1 - q : q;
-  const TileRef t = tile_ref(e.boundary_map, g);
+  const int32_t* src = reinterpret_cast<const int32_t*>(e.bdesc + g);
+  int32_t* dsc = desc_s[w];
+  const uint32_t mask = (uint32_t)__ldg(src + 32 + lane);
+  dsc[lane] = __ldg(src + lane);
+  __syncwarp();
+  const EnsBoundaryDesc& t = *reinterpret_cast<const EnsBoundaryDesc*>(dsc);  // up to `mask`
   const MemberDev& md = e.mem[t.member];
+  const DevLattice& d = md.d;
+  const EnsView v{reinterpret_cast<void*>(t.pop), t.np, reinterpret_cast<const uint32_t*>(t.slot_io),
+                  reinterpret_cast<const int32_t*>(t.seg_tab), d.n, d.slot_nbr, d.slot_prof, d.slot_F,
+                  d.slot_kappa, d.slot_dE, d.slot_Uw, d.slot_stride, d.iolets, d.err, d.chk};
   StepParams pm = p;
-  pm.omega = md.omega;
-  pm.omega_f = md.omega_f;
+  pm.omega_f = t.omega_f;
+  if constexpr (std::is_same<C, double>::value) pm.omega = md.omega;
   pm.rho0 = md.rho0;
   pm.rho0_f = md.rho0_f;
   pm.rho0_exact = md.rho0_exact;
   pm.diag = 0;  // ensembles: no fused diagnostics
-  pm.elastic = md.elastic;
-  pm.wall_uniform = md.wall_uniform;
+  pm.elastic = e.elastic_all >= 0 ? e.elastic_all : md.elastic;
+  pm.wall_uniform = e.uniform_all ? 1 : md.wall_uniform;
   pm.wall_F_f = md.wall_F_f;
   pm.wall_F = md.wall_F;
   pm.wall_K = md.wall_K;
-  boundary_tile<S, ODD>(md.d, pm, t.k, desc_s[w], stage[w], &bars[w], gs[w], lane);
+  boundary_tile<S, ODD, 0, false, true>(v, pm, t.k, dsc, stage[w], &bars[w], gs[w], lane, nullptr,
+                                        nullptr, nullptr, mask);
 }
 
 // ------------------------------------------------- persistent ensemble kernel
@@ -3068,6 +3132,13 @@ int launch_ens_desc(int storage, const MemberDev* mem, const TileRef* map, int64
   if (n <= 0) return 0;
   k_ens_desc<<<blocks_for(n * 32, 256), 256, 0, (cudaStream_t)stream>>>(
       mem, map, n, (int)storage_bytes(storage), out);
+  return (int)cudaGetLastError();
+}
+
+int launch_ens_bdesc(const MemberDev* mem, const TileRef* map, int64_t n, EnsBoundaryDesc* out,
+                     void* stream) {
+  if (n <= 0) return 0;
+  k_ens_bdesc<<<blocks_for(n * 32, 256), 256, 0, (cudaStream_t)stream>>>(mem, map, n, out);
   return (int)cudaGetLastError();
 }
 

@@ -274,6 +274,24 @@ struct alignas(16) EnsDesc {
 };
 static_assert(sizeof(EnsDesc) == 96, "EnsDesc must be 96 bytes");
 
+// A boundary tile of an ensemble with what its kernel needs before the
+// populations: the launch descriptor, the lanes' masks, and of its member the
+// address and row length of the populations, the bases of the iolet words and
+// segment tables, and 1 / tau; the member's other fields come from the table.
+struct alignas(16) EnsBoundaryDesc {
+  LaunchDesc launch;
+  uint64_t pop;
+  int32_t np;
+  int32_t member;
+  uint64_t slot_io;
+  uint64_t seg_tab;
+  int32_t k;  // launch position in the member
+  float omega_f;
+  int32_t pad[2];
+  uint32_t mask[kTile];
+};
+static_assert(sizeof(EnsBoundaryDesc) == 256, "EnsBoundaryDesc must be 256 bytes");
+
 // Ensemble launch: the members' bulk (boundary) tiles are numbered in
 // schedule order; bulk_map[g] (boundary_map[g]) names the member and launch
 // position of global bulk (boundary) tile g.
@@ -283,6 +301,10 @@ struct EnsembleLaunch {
   const TileRef* boundary_map;  // [n_boundary_tiles]
   const EnsDesc* desc;          // [n_desc] bulk tiles, each member's padded to an even number
   int64_t n_desc;
+  const EnsBoundaryDesc* bdesc;  // [n_boundary_tiles]
+  // wall model and uniform wall parameters when all members agree (launch
+  // constants: no load before the populations'), else -1 and 0
+  int32_t elastic_all, uniform_all;
   int32_t n_members;
   int64_t n_bulk_tiles, n_boundary_tiles;
   const MemberDev* multi_host;  // host copies of the members with multi-iolet tiles
@@ -317,6 +339,9 @@ int launch_small(int storage, const DevLattice& d, const StepParams& p, int64_t 
 // The descriptors of n bulk tiles (map: member and launch position, k < 0 for padding).
 int launch_ens_desc(int storage, const MemberDev* mem, const TileRef* map, int64_t n, EnsDesc* out,
                     void* stream);
+// The descriptors of the ensemble's n boundary tiles (map: member and launch position).
+int launch_ens_bdesc(const MemberDev* mem, const TileRef* map, int64_t n, EnsBoundaryDesc* out,
+                     void* stream);
 int launch_advance(int64_t* step_dev, int64_t by, void* stream);
 int launch_set_step(int64_t* step_dev, int64_t value, void* stream);
 int launch_init(int storage, const DevLattice& d, const double* rho, const double* u,
