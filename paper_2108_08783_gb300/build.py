@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblbm.so")
 BUILD = os.path.join(HERE, "_build")
 SOURCES = ["lattice_build.cpp", "kernels.cu", "capi.cu", "mlp.cu"]
-HEADERS = ["lbm_internal.h", "d3q19.h", "mlp_fused.cuh"]
+HEADERS = ["lbm_internal.h", "d3q19.h", "mlp_fused.cuh", "warm_frame.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 

@@ -1717,26 +1717,19 @@ int lbm_warm_start(lbm_ctx* c, lbm_mlp* net, const lbm_warm_frame* frame) {
   // queued work finish first.
   cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(ns));
   if (e != cudaSuccess) return cuda_fail(c, e, "lbm_warm_start: network stream");
-  const size_t n = (size_t)c->L.n;
-  Temp tx(c, n * n_in * sizeof(float)), ty(c, n * 3 * sizeof(float));
-  Temp tr(c, n * sizeof(double)), tu(c, 3 * n * sizeof(double));
-  if (!tx.p || !ty.p || !tr.p || !tu.p) return fail(c, LBM_ENOMEM, "lbm_warm_start: allocation");
-  rc = check_launch(c, lbm::launch_warm_features(c->coords_dev, (int64_t)n, f, nullptr, nullptr,
-                                                 (float*)tx.p, nullptr, c->stream),
+  const int64_t n = c->L.n;
+  Temp tx(c, (size_t)n * n_in * sizeof(float)), ty(c, (size_t)n * 3 * sizeof(float));
+  if (!tx.p || !ty.p) return fail(c, LBM_ENOMEM, "lbm_warm_start: allocation");
+  float* x = static_cast<float*>(tx.p);
+  float* y = static_cast<float*>(ty.p);
+  rc = check_launch(c, lbm::launch_warm_features(c->coords_dev, n, f, nullptr, nullptr, x, nullptr,
+                                                 c->stream),
                     "warm feature kernel");
   if (rc == LBM_OK)
-    rc = check_launch(c, lbm::mlp_forward_on(net, (const float*)tx.p, (int64_t)n, (float*)ty.p,
-                                             c->stream),
-                      "network forward");
+    rc = check_launch(c, lbm::mlp_forward_on(net, x, n, y, c->stream), "network forward");
   if (rc == LBM_OK)
-    rc = check_launch(c, lbm::launch_warm_fields(c->coords_dev, (int64_t)n, f,
-                                                 (const float*)ty.p, (double*)tr.p,
-                                                 (double*)tu.p, c->stream),
-                      "warm field kernel");
-  if (rc == LBM_OK)
-    rc = check_launch(c, lbm::launch_init(c->storage, c->d, (double*)tr.p, (double*)tu.p,
-                                          c->stream),
-                      "init kernel");
+    rc = check_launch(c, lbm::launch_warm_init(c->storage, c->d, c->coords_dev, f, y, c->stream),
+                      "warm population kernel");
   const int rs = sync(c, "lbm_warm_start");
   if (rc == LBM_OK) rc = rs;
   if (rc == LBM_OK) c->step = 0;

@@ -371,13 +371,15 @@ int launch_check_counts(const DevLattice& d, void* stream);
 
 // Learned warm start (mlp.cu): the network's forward pass on a given stream
 // (n rows in chunks of its batch size, using its activation buffers), its
-// shape and stream, and the per-site feature / field kernels.
+// shape and stream, and the per-site kernels:
 int mlp_forward_on(lbm_mlp* net, const float* x, int64_t n, float* y, void* stream);
 void mlp_shape(const lbm_mlp* net, int* n_in, int* n_out, void** stream);
+// features, and populations at equilibrium with the fields the outputs y stand
+// for (kernels.cu).
 int launch_warm_features(const int32_t* coords, int64_t n, const lbm_warm_frame& f,
                          const double* rho, const double* u, float* x, float* t, void* stream);
-int launch_warm_fields(const int32_t* coords, int64_t n, const lbm_warm_frame& f, const float* y,
-                       double* rho, double* u, void* stream);
+int launch_warm_init(int storage, const DevLattice& d, const int32_t* coords,
+                     const lbm_warm_frame& f, const float* y, void* stream);
 
 int reduce_partials();
 
