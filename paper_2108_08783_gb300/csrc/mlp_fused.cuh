@@ -374,8 +374,13 @@ struct TrainArgs {
   double* loss_part;        // [tiles][4]
 };
 
+// Waits see a phase by its parity only, so no barrier may run two phases ahead
+// of a thread that waits on it.  `ready` (a product's operand is staged) and
+// `acc` (it is computed) alternate; delta_0, which no product follows, has a
+// barrier of its own: on `ready` the next tile's inputs could complete a second
+// phase before the product warp had seen the first, and it would wait for ever.
 struct TrainBars {
-  uint64_t w_full, acc, ready;
+  uint64_t w_full, acc, ready, tail;
   uint32_t tmem;
 };
 
@@ -398,6 +403,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     mbar_init_n(&s.w_full, 1);
     mbar_init_n(&s.acc, 1);
     mbar_init_n(&s.ready, kTrainEpiWarps * 32);
+    mbar_init_n(&s.tail, kTrainEpiWarps * 32);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc_before();
@@ -436,7 +442,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   } else if (warp == kTrainEpiWarps + 1) {
     if (lane == 0) {
       bool ok = true;
-      uint32_t rd = 0, wf = 0;
+      uint32_t rd = 0, wf = 0, tl = 0;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         for (int g = 0; g < ops; ++g) {
           ok = mbar_wait(&s.ready, rd++ & 1u) && mbar_wait(&s.w_full, wf++ & 1u);
@@ -467,7 +473,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
           copy_s2g((fwd ? a.h[l] : a.d[l]) + t * bytes, b, bytes);
         }
         // delta_0, ready after the last product's epilogue
-        if (ok) ok = mbar_wait(&s.ready, rd++ & 1u);
+        if (ok) ok = mbar_wait(&s.tail, tl++ & 1u);
         if (ok) {
           const uint32_t bytes = (uint32_t)net.l[0].rg * kstr;
           copy_s2g(a.d[0] + t * bytes, image(1), bytes);
@@ -488,16 +494,16 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       tc_after();
       return ok;
     };
-    auto publish = [&]() {
+    auto publish = [&](uint64_t* bar) {
       fence_async();
       tc_before();
-      mbar_arrive(&s.ready);
+      mbar_arrive(bar);
     };
     for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int64_t row0 = t * nb;
       const int valid = (int)(a.n - row0 < nb ? a.n - row0 : nb);
       stage_inputs(image(0), a.x, row0, valid, net.n_in, nb, tid, kTrainEpiWarps * 32);
-      publish();
+      publish(&s.ready);
       // hidden layers: two accumulator tiles, two warps of 8-row column groups
       // each (one tile: four)
       const bool two = net.l[0].rg > 16;
@@ -520,7 +526,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
             w[j] = bf16_pair(tanhf(v[2 * j] + bias), tanhf(v[2 * j + 1] + bias));
           *reinterpret_cast<uint4*>(row + c * kCoreBytes) = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        publish();
+        publish(&s.ready);
       }
       if (!ok) break;
       // output layer: y, the loss and its error delta_{L-1} = 2 (y - t) / count
@@ -561,7 +567,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
           for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
           if (lane == 0) a.loss_part[t * 4 + quarter] = (double)sum * a.inv_count;
         }
-        publish();
+        publish(&s.ready);
       }
       // way back: delta_{l-1} = (delta_l W_l)(1 - h_l^2) over h_l
       for (int l = NL - 1; l >= 1 && ok; --l) {
@@ -582,7 +588,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
           }
           *p = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        publish();
+        publish(l > 1 ? &s.ready : &s.tail);
       }
     }
     if (!ok && lane == 0) atomicOr(net.err, 1);
