@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm(const GemmArgs g) {
     for (int c0 = 0; c0 < kTN; c0 += 16) {
       uint32_t v[16];
       const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+      __syncwarp();  // lanes of rows beyond M went ahead: the load is collective
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
           "%13,%14,%15}, [%16];"

@@ -111,8 +111,11 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
       "l"(a), "l"(b), "r"(idesc), "r"(acc ? 1u : 0u)
       : "memory");
 }
+// The loads are collective (.sync.aligned): the warp is brought together first,
+// as loops issue them after branches by lane.
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&v)[8]) {
   uint32_t r[8];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
@@ -124,6 +127,7 @@ __device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&v)[8]) {
 }
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
       "%13,%14,%15}, [%16];"

@@ -41,3 +41,27 @@ def test_gradient_over_several_tiles_per_cta(shape):
         loss2, g2 = net.loss_grad(xd, td)
         net.sync()
         assert loss2 == loss and np.array_equal(g, g2)
+
+
+@pytest.mark.parametrize("width", [48, 100, 208, 272])
+def test_widths_that_end_inside_a_warp(width):
+    """Half of a warp's lanes leave the epilogue's stores out before the next
+    collective load from tensor memory (272: the layer-by-layer kernel, whose
+    rows beyond the batch do)."""
+    import torch
+    from paper_2108_08783_gb300 import MLP
+    n = 177
+    net = MLP(5, width, 3, 9, max_batch=n)
+    theta = I.mlp_init(3, 5, width, 3, 9, bias_scale=0.1)
+    net.set_params(theta)
+    x, t = I.mlp_batch(4, n, 5, 9, scale=0.5)
+    sizes = M.layer_sizes(5, width, 3, 9)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    y = net.forward(xd)
+    loss, g = net.loss_grad(xd, td)
+    net.sync()
+    y_ref, _ = M.forward(theta, sizes, x, bf16=True)
+    E, g_ref = M.loss_grad(theta, sizes, x, t, bf16=True)
+    assert np.linalg.norm(y.cpu().numpy() - y_ref) < 2e-3 * np.linalg.norm(y_ref)
+    assert abs(loss - E) <= 1e-3 * E
+    assert np.linalg.norm(np.asarray(g, np.float64) - g_ref) < 1e-2 * np.linalg.norm(g_ref)
