@@ -327,22 +327,26 @@ __device__ __forceinline__ Mom<C> moments(const C (&g)[kQ]) {
 // Two forms; in both every operation is written out (nothing is left to the
 // compiler to contract), so that all kernels round alike.
 //
-// Plain (FP32 storage, and every boundary tile): 9 operations a pair beyond cu,
-// where adding and subtracting the odd part took 10. The coefficients are one
-// rounding away from rho and drho, as rounding errors they share are not
+// Plain (FP64 and FP32 storage, and every boundary tile): 9 operations a pair
+// beyond cu, where adding and subtracting the odd part took 10. The coefficients
+// are one rounding away from rho and drho, as rounding errors they share are not
 // averaged out over the directions: the scaled form below left the fields of
 // FP32 runs 1.3 to 1.5 times further from FP64.
-// Scaled (16-bit storage, whose rounding is 2^13 times coarser, and FP64, where
-// the operations are what a site costs): omega and the weights multiplied into
+// Scaled (16-bit storage, whose rounding is 2^13 times coarser): omega and the
+// weights multiplied into
 //   omega g^eq = k + h cu^2 +- l cu,  k = omega w (drho - 1.5 rho u.u),
 //   h = 4.5 omega w rho,  l = 3 omega w rho,  g* = (1 - omega) g + omega g^eq:
 // 6 operations a pair.
 // The coefficients are those of the axis directions (w = 1/18); next() halves
-// them (exactly) for the diagonals. Every weight is a multiple of the FP32
-// 1/18 (7e-9 off): 1/6 for the odd part or 1/3 for the rest population, 3e-8
-// off, would change the momentum or the mass by the same fraction at every
-// step, and were the larger part of the error of FP32 runs (40 steps of the
-// long tube: 1.2e-6 to 1.7e-6 before, 0.6e-6 so).
+// them (exactly) for the diagonals. In the plain form every weight is a multiple
+// of the FP32 1/18 (7e-9 off): 1/6 for the odd part or 1/3 for the rest
+// population, 3e-8 off, would change the momentum or the mass by the same
+// fraction at every step, and were the larger part of the error of FP32 runs (40
+// steps of the long tube: 1.2e-6 to 1.7e-6 before, 0.6e-6 so). The scaled form's
+// h is off that multiple, so that a step adds 18 fl(1/18) - 1 of omega rho 1.5 u.u
+// to a site's mass: nothing beside 16-bit rounding, but 30 times the drift of
+// the plain form in FP64 (tests/test_gpu_mass.py), whose density after 300
+// steps of a decaying flow was 2 to 7 times further off.
 template <class C, bool SCALED>
 struct Relax;
 template <class C>
@@ -580,7 +584,7 @@ __device__ __forceinline__ typename Codec<S>::C bulk_update(S* P, int64_t np, in
     if ((threadIdx.x & 31) == 0) *slot = (double)sum;
   }
   if (unstable(m.rho)) atomicOr(err_word(err), kErrUnstable);
-  Relax<C, !std::is_same<S, float>::value> rx(m, omega);
+  Relax<C, sizeof(S) == 2> rx(m, omega);
   const StoreBase<S, ODD, E> B(P, np);
   Cd::st(B.q + x, 0, rx.rest(m, g[0]));
   chk_count(chk, P, P + x, kQ * np, err);
