@@ -422,6 +422,7 @@ int lbm_build_lattice(const uint8_t* labels, int32_t nx, int32_t ny, int32_t nz,
     t.phase_inc = lbm::frac_to_u64(inv - std::floor(inv));
     const double ph = t.phase * (0.5 / M_PI);
     t.phase_off = lbm::frac_to_u64(ph - std::floor(ph));
+    lbm::fixed_phase(t.period, t.phase, &t.inc_hi, &t.inc_lo, &t.off64);
     t.rho_f = (float)t.rho;
     t.drho_f = (float)(t.rho - 1.0);
     t.u_mean_f = (float)t.u_mean;

@@ -212,20 +212,23 @@ __device__ __forceinline__ float omega_as<float>(double, float wf) { return wf; 
 
 // Velocity inlet (Sec. 3) of a site with profile values (p0, ps, pc) at step
 // n: u_in = axis (u_mean p0 + u_amp (ps sin th + pc cos th)),
-// th = 2 pi n / T + phase, from the iolet's 64-bit fixed-point phase
-// (frac(n / T + phase / 2 pi) in integer arithmetic, exact modulo one period).
-// FP64 paths keep its top 53 bits (7e-16 rad, as exact as 2 pi n / T + phase
-// rounded to FP64, which loses more the larger n is) and take sinpi and cospi in
-// FP64: no range reduction, which with sin and cos of th was a third of the FP64
-// operations of an inlet tile.  FP32 paths keep 24 bits (a phase error below
-// 2^-24 of a period, ~4e-7 rad) and evaluate sinpi/cospi and the profile in FP32.
+// th = 2 pi n / T + phase, from the iolet's fixed-point phase: frac(n / T +
+// phase / 2 pi) in units of 2^-64, integer arithmetic modulo one period.
+// FP64 paths take 1 / T to 2^-128, so the phase is right to 2^-64 of a period at
+// any step, and its nearest FP64 number in [-1, 1) half periods: 2e-16 rad at
+// most, where 2 pi n / T + phase rounded to FP64 loses more the larger n is.
+// sinpi and cospi of it need no range reduction, which with sin and cos of th
+// was a third of the FP64 operations of an inlet tile.  FP32 paths keep 24 bits
+// of a 64-bit increment's phase (an error below 2^-24 of a period, ~4e-7 rad)
+// and evaluate sinpi/cospi and the profile in FP32.
 __device__ __forceinline__ void inlet_velocity(const IoletDev& io, int64_t n, double p0, double ps,
                                                double pc, double& ux, double& uy, double& uz) {
   double g = mul_pin(io.u_mean, p0);
   if (!io.steady) {
     double sn, cs;
-    const uint64_t ph = io.phase_off + (uint64_t)n * io.phase_inc;  // mod 2^64
-    sincospi(__fma_rn((double)(ph >> 11), 0x1p-52, io.finite), &sn, &cs);
+    const uint64_t ph =
+        io.off64 + (uint64_t)n * io.inc_hi + __umul64hi((uint64_t)n, io.inc_lo);  // mod 2^64
+    sincospi(__fma_rn((double)(int64_t)ph, 0x1p-63, io.finite), &sn, &cs);
     g = fma_pin(io.u_amp, fma_pin(ps, sn, mul_pin(pc, cs)), g);
   }
   ux = mul_pin(g, io.axis[0]);

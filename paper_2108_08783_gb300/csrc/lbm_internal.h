@@ -90,6 +90,11 @@ struct IoletDev {
   // copies of rho, rho - 1, u_mean, u_amp and the axis.
   uint64_t phase_inc;
   uint64_t phase_off;
+  // The same for the FP64 paths: 1 / T to 2^-128 (inc_hi inc_lo), so that no
+  // drift n 2^-64 of a truncated increment adds up over a long run.
+  uint64_t inc_hi, inc_lo;
+  uint64_t off64;
+  uint64_t pad64;
   float rho_f, drho_f, u_mean_f, u_amp_f;
   float axis_f[3];
   float pad_f;
@@ -100,6 +105,28 @@ static_assert(sizeof(IoletDev) % 16 == 0, "IoletDev alignment");
 inline uint64_t frac_to_u64(double x) {
   if (!(x >= 0.0) || x >= 1.0) return 0;
   return (uint64_t)std::ldexp(x, 64);
+}
+
+// 2^128 x modulo 2^128 for |x| < 1 (two's complement; anything else gives 0).
+inline unsigned __int128 frac_to_u128(double x) {
+  if (!(x > -1.0 && x < 1.0) || x == 0.0) return 0;
+  int e;
+  const double m = std::frexp(std::fabs(x), &e);  // m in [0.5, 1)
+  unsigned __int128 v = (uint64_t)std::ldexp(m, 53);
+  const int sh = 75 + e;
+  v = sh >= 0 ? v << sh : (sh > -64 ? v >> -sh : 0);
+  return x < 0.0 ? (unsigned __int128)0 - v : v;
+}
+// frac(1 / T) in units of 2^-128 and frac(phase / 2 pi) in units of 2^-64, from
+// quotient and product with their remainders.
+inline void fixed_phase(double T, double phase, uint64_t* hi, uint64_t* lo, uint64_t* off) {
+  const double q = 1.0 / T, qr = std::fma(-q, T, 1.0) / T;
+  const unsigned __int128 inc = frac_to_u128(q - std::trunc(q)) + frac_to_u128(qr);
+  *hi = (uint64_t)(inc >> 64);
+  *lo = (uint64_t)inc;
+  const double c0 = 0x1.45f306dc9c883p-3, c1 = -0x1.6b01ec5417056p-57;  // 1 / 2 pi
+  const double a = phase * c0, ar = std::fma(phase, c0, -a) + phase * c1;
+  *off = (uint64_t)((frac_to_u128(a - std::trunc(a)) + frac_to_u128(ar)) >> 64);
 }
 
 // Allocator whose resize() leaves new elements uninitialised, for the large
