@@ -354,9 +354,10 @@ int lbm_fmap(const double *alpha, int64_t n_alpha, const double *dr_over_R, int6
  * (the first use builds the tensor map of the population array; the same
  * results as 2, bit for bit).  Defaults are chosen per storage at build
  * time.  A lattice of at most 16 tiles per SM takes all steps of an lbm_step
- * call in one launch (the same results) until a knob is set: then it takes the
- * launches the knobs describe.  LBM_EINVAL for another knob or value, LBM_ECUDA when the tensor map
- * cannot be made. */
+ * call in one launch (the same results) while every knob has its default, and
+ * the launches the knobs describe when one has not.  LBM_EINVAL for another
+ * knob or value (nothing changes), LBM_ECUDA when the tensor map cannot be
+ * made. */
 int lbm_tune(lbm_ctx *ctx, int32_t knob, int64_t value);
 
 /* lbm_set_stream - run subsequent work on another cudaStream_t. */

@@ -92,10 +92,9 @@ struct lbm_ctx {
   // compile-time offset (the parity plus the step within the block)
   int64_t* step_d = nullptr;
   int64_t step_d_for = -1;
-  // small lattices: all steps of a call in one cooperative launch (k_small),
-  // unless a launch knob has been set
+  // small lattices: all steps of a call in one cooperative launch (k_small)
+  // while every launch knob has its default (default_knobs)
   bool small = false;
-  bool tuned = false;
   unsigned long long* small_bar = nullptr;
   // tensor map of the populations as a [19][npad] array of 16-bit elements,
   // boxes of 32 x 19 (staged-row bulk kernel), made on first use
@@ -135,6 +134,14 @@ namespace {
 // Steps per captured graph of a lattice by default: +3 % on the long tube
 // against direct launches (100 gains another 0.1-0.4 %).
 constexpr int64_t kDefaultGraphSteps = 20;
+constexpr int32_t kDefaultBulkWarps = 4;
+
+// Every launch knob of lbm_tune has the value it had at build.
+bool default_knobs(const lbm_ctx* c) {
+  return c->prefetch == default_prefetch(c->storage) &&
+         c->bulk_sites == default_bulk_sites(c->storage) && c->bulk_warps == kDefaultBulkWarps &&
+         c->graph_steps == kDefaultGraphSteps;
+}
 
 // Steps per launch of the small-lattice kernel (some milliseconds).
 constexpr int64_t kSmallSteps = 1000;
@@ -635,7 +642,7 @@ bool capturing(cudaStream_t s) {
 int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
   lbm::StepParams p = step_params(c);
 #ifndef LBM_CHECKED
-  if (c->small && !c->tuned && !diag_last && !c->prof && n_steps > 0 && !capturing(c->stream)) {
+  if (c->small && default_knobs(c) && !diag_last && !c->prof && n_steps > 0 && !capturing(c->stream)) {
     for (int64_t done = 0; done < n_steps;) {
       const int64_t m = std::min(n_steps - done, kSmallSteps);
       p.step = c->step;
@@ -867,7 +874,6 @@ int lbm_tune(lbm_ctx* c, int32_t knob, int64_t value) {
   if (!c) return LBM_EINVAL;
   c->err.clear();
   c->gexec_steps[0] = c->gexec_steps[1] = 0;  // captured steps hold the old settings
-  c->tuned = true;     // the launches asked for, whatever the size
   switch (knob) {
     case LBM_TUNE_GRAPH_STEPS:
       if (value < 0 || (value & 1)) return fail(c, LBM_EINVAL, "graph steps must be even and >= 0");

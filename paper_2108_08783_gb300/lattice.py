@@ -297,7 +297,8 @@ class Lattice:
     def tune(self, prefetch=None, bulk_sites=None, bulk_warps=None, graph_steps=None):
         """Launch knobs (``lbm_tune``): L2 prefetch distance of the bulk kernel in
         tiles, the bulk kernel's sites per lane and their pairing (1 to 4), and
-        its warps per CTA (4 or 8)."""
+        its warps per CTA (4 or 8).  A small lattice takes all steps of a call in
+        one launch while all of them have their defaults."""
         if prefetch is not None:
             self._check(self._lib.lbm_tune(self.h, A.LBM_TUNE_PREFETCH, int(prefetch)))
         if bulk_sites is not None:
@@ -326,7 +327,8 @@ class Lattice:
         two tiles), its CTA size, its L2 prefetch distance and graph replay by
         timing each candidate on this lattice (``coordinate_search`` from the
         library's defaults, sites per lane and prefetch distance jointly;
-        ``trials`` and ``sweeps`` as there).  Every trial, and the warm-up run
+        ``trials`` and ``sweeps`` as there).  On a small lattice the defaults are
+        its one launch for all steps.  Every trial, and the warm-up run
         before each candidate's trials, advances the lattice by ``trial_steps``
         steps (an even number keeps both parities equal)."""
         if self.storage == "f64":
