@@ -643,15 +643,20 @@ int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
   lbm::StepParams p = step_params(c);
 #ifndef LBM_CHECKED
   if (c->small && default_knobs(c) && !diag_last && !c->prof && n_steps > 0 && !capturing(c->stream)) {
-    for (int64_t done = 0; done < n_steps;) {
-      const int64_t m = std::min(n_steps - done, kSmallSteps);
+    while (n_steps > 0) {
+      const int64_t m = std::min(n_steps, kSmallSteps);
       p.step = c->step;
-      const int lr = lbm::launch_small(c->storage, c->d, p, m, c->small_bar, c->stream);
-      if (lr != 0) return cuda_fail(c, (cudaError_t)lr, "step kernel");
+      if (lbm::launch_small(c->storage, c->d, p, m, c->small_bar, c->stream) != 0) {
+        // refused (a stream with fewer SMs, say): nothing ran, and the launched
+        // kernels below take the rest; an error they share comes back from them
+        cudaGetLastError();
+        c->small = false;
+        break;
+      }
       c->step += m;
-      done += m;
+      n_steps -= m;
     }
-    return LBM_OK;
+    if (n_steps == 0) return LBM_OK;
   }
   const int64_t G = c->graph_steps;
   if (G > 0 && n_steps >= G && !diag_last && !c->prof) {

@@ -3136,10 +3136,15 @@ int64_t small_tiles(int storage, int n_sms) {
     using S = std::remove_pointer_t<decltype(tag)>;
     using Cfg = SmallCfg<S>;
     const int bytes = Cfg::warps * Cfg::per_warp;
-    const int r = (int)cudaFuncSetAttribute(k_small<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            bytes);
-    tiles = (int64_t)n_sms * Cfg::warps;
-    return r;
+    int dev = 0, coop = 0, per_sm = 0;
+    cudaError_t r = cudaFuncSetAttribute(k_small<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         bytes);
+    if (r == cudaSuccess) r = cudaGetDevice(&dev);
+    if (r == cudaSuccess) r = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (r == cudaSuccess)
+      r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_small<S>, Cfg::warps * 32, bytes);
+    if (coop && per_sm >= 1) tiles = (int64_t)n_sms * Cfg::warps;  // the grid is one CTA per SM
+    return (int)r;
   });
   if (e != 0) {
     cudaGetLastError();
