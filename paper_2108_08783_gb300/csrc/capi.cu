@@ -1276,7 +1276,8 @@ struct lbm_ensemble {
   std::vector<cudaStream_t> member_streams;  // distinct streams of the members
   std::vector<void*> owned;       // device buffers (member 0's allocator)
   lbm::MemberDev* mem_d = nullptr;
-  lbm::TileRef* map_d = nullptr;  // tile maps: bulk tiles, then boundary tiles
+  // tile maps: bulk tiles, boundary tiles, then the bulk tiles padded (desc_d's)
+  lbm::TileRef* map_d = nullptr;
   lbm::EnsDesc* desc_d = nullptr;  // bulk tile descriptors, members padded to even numbers
   int64_t n_desc = 0;
   lbm::EnsBoundaryDesc* bdesc_d = nullptr;  // boundary tile descriptors
@@ -1294,6 +1295,7 @@ struct lbm_ensemble {
   int64_t exec_steps = 0;
   int exec_parity = -1;
   lbm::EnsembleLaunch launch{};
+  std::vector<lbm::MemberDev> tab_host;    // the member table as uploaded
   std::vector<lbm::MemberDev> multi_host;  // members with multi-iolet tiles (host copies)
   std::string err;
 };
@@ -1318,18 +1320,25 @@ void ens_drop_graph(lbm_ensemble* e) {
   e->exec_parity = -1;
 }
 
-// Upload the member table and the prefix tables in schedule order.
 // Tile maps in schedule order: for every global bulk (boundary) tile, its
-// member's position in the member table and its launch position there.
-int ens_maps(lbm_ensemble* e) {
+// member's position in the member table and its launch position there; and the
+// bulk tiles again with each member's padded to an even number. The one host
+// allocation of a change of schedule comes first: without it (std::bad_alloc)
+// nothing has changed.
+int ens_maps(lbm_ensemble* e, const std::vector<int32_t>& order) {
   const int n = (int)e->members.size();
-  std::vector<lbm::TileRef> map((size_t)(e->n_bulk + e->n_boundary));
-  size_t gb = 0, gd = (size_t)e->n_bulk;
+  std::vector<lbm::TileRef> map((size_t)(e->n_bulk + e->n_boundary + e->n_desc));
+  size_t gb = 0, gd = (size_t)e->n_bulk, gp = (size_t)(e->n_bulk + e->n_boundary);
   for (int q = 0; q < n; ++q) {
-    const lbm_ctx* c = e->members[e->order[q]];
-    for (int64_t k = c->d.n_boundary; k < c->d.n_tiles; ++k) map[gb++] = lbm::TileRef{q, (int32_t)k};
+    const lbm_ctx* c = e->members[order[q]];
     for (int64_t k = 0; k < c->d.n_boundary; ++k) map[gd++] = lbm::TileRef{q, (int32_t)k};
+    for (int64_t k = c->d.n_boundary; k < c->d.n_tiles; ++k) {
+      map[gb++] = lbm::TileRef{q, (int32_t)k};
+      map[gp++] = lbm::TileRef{q, (int32_t)k};
+    }
+    if ((c->d.n_tiles - c->d.n_boundary) & 1) map[gp++] = lbm::TileRef{q, -1};
   }
+  e->order = order;
   cudaError_t r = cudaMemcpyAsync(e->map_d, map.data(), map.size() * sizeof(lbm::TileRef),
                                   cudaMemcpyHostToDevice, e->stream);
   if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);  // map is a temporary
@@ -1340,9 +1349,10 @@ int ens_maps(lbm_ensemble* e) {
   return LBM_OK;
 }
 
+// Upload the member table in schedule order.
 int ens_upload(lbm_ensemble* e) {
   const int n = (int)e->members.size();
-  std::vector<lbm::MemberDev> tab(n);
+  std::vector<lbm::MemberDev>& tab = e->tab_host;
   for (int q = 0; q < n; ++q) {
     const lbm_ctx* c = e->members[e->order[q]];
     lbm::MemberDev& md = tab[q];
@@ -1362,7 +1372,7 @@ int ens_upload(lbm_ensemble* e) {
   }
   cudaError_t r = cudaMemcpyAsync(e->mem_d, tab.data(), n * sizeof(lbm::MemberDev),
                                   cudaMemcpyHostToDevice, e->stream);
-  if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);  // tab is a temporary
+  if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);  // tab is written again
   if (r != cudaSuccess) return ens_cuda(e, r, "ensemble upload");
   e->multi_host.clear();
   for (const lbm::MemberDev& md : tab)
@@ -1387,33 +1397,25 @@ int ens_upload(lbm_ensemble* e) {
 }
 
 // The tiles' descriptors in schedule order, from the members' launch lists
-// (after ens_maps and ens_upload: the kernels read the tile map and the member table).
+// (after ens_maps and ens_upload: the kernels read the tile maps and the member table).
 int ens_descs(lbm_ensemble* e) {
-  cudaError_t rb = (cudaError_t)lbm::launch_ens_bdesc(e->mem_d, e->launch.boundary_map,
-                                                      e->n_boundary, e->bdesc_d, e->stream);
-  if (rb != cudaSuccess) return ens_cuda(e, rb, "ensemble descriptors");
-  if (e->n_desc == 0) {
-    rb = cudaStreamSynchronize(e->stream);
-    return rb == cudaSuccess ? LBM_OK : ens_cuda(e, rb, "ensemble descriptors");
-  }
-  std::vector<lbm::TileRef> map;
-  map.reserve((size_t)e->n_desc);
-  for (int q = 0; q < (int)e->members.size(); ++q) {
-    const lbm_ctx* c = e->members[e->order[q]];
-    for (int64_t k = c->d.n_boundary; k < c->d.n_tiles; ++k) map.push_back(lbm::TileRef{q, (int32_t)k});
-    if (map.size() & 1) map.push_back(lbm::TileRef{q, -1});
-  }
-  Temp t(e->members[0], map.size() * sizeof(lbm::TileRef));
-  if (!t.p) return ens_fail(e, LBM_ENOMEM, "ensemble descriptors: allocation");
-  cudaError_t r = cudaMemcpyAsync(t.p, map.data(), map.size() * sizeof(lbm::TileRef),
-                                  cudaMemcpyHostToDevice, e->stream);
+  cudaError_t r = (cudaError_t)lbm::launch_ens_bdesc(e->mem_d, e->launch.boundary_map,
+                                                     e->n_boundary, e->bdesc_d, e->stream);
   if (r == cudaSuccess)
-    r = (cudaError_t)lbm::launch_ens_desc(e->storage, e->mem_d, static_cast<lbm::TileRef*>(t.p),
-                                          (int64_t)map.size(), e->desc_d, e->stream);
-  const cudaError_t r2 = cudaStreamSynchronize(e->stream);  // the maps are temporaries
-  if (r == cudaSuccess) r = r2;
+    r = (cudaError_t)lbm::launch_ens_desc(e->storage, e->mem_d, e->map_d + e->n_bulk + e->n_boundary,
+                                          e->n_desc, e->desc_d, e->stream);
+  if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);
   if (r != cudaSuccess) return ens_cuda(e, r, "ensemble descriptors");
   return LBM_OK;
+}
+
+// Number the members' tiles in another order. No device memory is allocated, so
+// what can fail half-way is a CUDA call only.
+int ens_schedule(lbm_ensemble* e, const std::vector<int32_t>& order) {
+  int rc = ens_maps(e, order);
+  if (rc == LBM_OK) rc = ens_upload(e);
+  if (rc == LBM_OK) rc = ens_descs(e);
+  return rc;
 }
 
 }  // namespace
@@ -1459,8 +1461,6 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
     if (std::find(e->member_streams.begin(), e->member_streams.end(), c->stream) ==
         e->member_streams.end())
       e->member_streams.push_back(c->stream);
-  e->order.resize(n);
-  for (int q = 0; q < n; ++q) e->order[q] = q;
   int lo = 0, hi = 0;
   cudaError_t r = cudaDeviceGetStreamPriorityRange(&lo, &hi);
   if (r == cudaSuccess) r = cudaStreamCreateWithFlags(&e->stream, cudaStreamNonBlocking);
@@ -1485,7 +1485,7 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
   }
   e->mem_d = static_cast<lbm::MemberDev*>(alloc(n * sizeof(lbm::MemberDev)));
   e->map_d = static_cast<lbm::TileRef*>(
-      alloc(std::max<int64_t>(1, e->n_bulk + e->n_boundary) * sizeof(lbm::TileRef)));
+      alloc(std::max<int64_t>(1, e->n_bulk + e->n_boundary + e->n_desc) * sizeof(lbm::TileRef)));
   e->desc_d = static_cast<lbm::EnsDesc*>(
       alloc(std::max<int64_t>(1, e->n_desc) * sizeof(lbm::EnsDesc)));
   e->bdesc_d = static_cast<lbm::EnsBoundaryDesc*>(
@@ -1496,9 +1496,16 @@ int lbm_ensemble_create(lbm_ctx* const* members, int32_t n, lbm_ensemble** out) 
     lbm_ensemble_destroy(e);
     return LBM_ENOMEM;
   }
-  int rc = ens_maps(e);
-  if (rc == LBM_OK) rc = ens_upload(e);
-  if (rc == LBM_OK) rc = ens_descs(e);
+  int rc;
+  try {
+    e->tab_host.resize((size_t)n);
+    e->multi_host.reserve((size_t)n);
+    std::vector<int32_t> order((size_t)n);
+    for (int q = 0; q < n; ++q) order[(size_t)q] = q;
+    rc = ens_schedule(e, order);
+  } catch (const std::bad_alloc&) {
+    rc = LBM_ENOMEM;
+  }
   if (rc != LBM_OK) {
     lbm_ensemble_destroy(e);
     return rc;
@@ -1517,19 +1524,20 @@ int lbm_ensemble_tune(lbm_ensemble* e, int32_t knob, int64_t value) {
       ens_drop_graph(e);
       return LBM_OK;
     case LBM_TUNE_SCHEDULE: {
-      const int n = (int)e->members.size();
-      for (int q = 0; q < n; ++q) e->order[q] = q;
-      if (value == 1) {  // largest members first
-        std::stable_sort(e->order.begin(), e->order.end(), [&](int a, int b) {
-          return e->members[a]->d.n_tiles > e->members[b]->d.n_tiles;
-        });
-      } else if (value != 0) {
+      if (value != 0 && value != 1)
         return ens_fail(e, LBM_EINVAL, "schedule must be 0 (given order) or 1 (largest first)");
+      try {
+        const int n = (int)e->members.size();
+        std::vector<int32_t> order((size_t)n);
+        for (int q = 0; q < n; ++q) order[(size_t)q] = q;
+        if (value == 1)  // largest members first
+          std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+            return e->members[a]->d.n_tiles > e->members[b]->d.n_tiles;
+          });
+        return ens_schedule(e, order);
+      } catch (const std::bad_alloc&) {
+        return ens_fail(e, LBM_ENOMEM, "schedule: host allocation");
       }
-      int rc = ens_maps(e);
-      if (rc == LBM_OK) rc = ens_upload(e);
-      if (rc == LBM_OK) rc = ens_descs(e);
-      return rc;
     }
     case LBM_TUNE_GRAPH_STEPS:
       if (value < 0 || (value & 1)) return ens_fail(e, LBM_EINVAL, "graph steps must be even");
