@@ -641,8 +641,14 @@ bool capturing(cudaStream_t s) {
 
 int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
   lbm::StepParams p = step_params(c);
-#ifndef LBM_CHECKED
-  if (c->small && default_knobs(c) && !diag_last && !c->prof && n_steps > 0 && !capturing(c->stream)) {
+  // (checked builds cover both paths: single steps take the launched kernels)
+#ifdef LBM_CHECKED
+  const int64_t small_from = 2;
+#else
+  const int64_t small_from = 1;
+#endif
+  if (c->small && default_knobs(c) && !diag_last && !c->prof && n_steps >= small_from &&
+      !capturing(c->stream)) {
     while (n_steps > 0) {
       const int64_t m = std::min(n_steps, kSmallSteps);
       p.step = c->step;
@@ -653,11 +659,16 @@ int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
         c->small = false;
         break;
       }
+#ifdef LBM_CHECKED
+      const int cr = lbm::launch_check_counts(c->d, (int)m, c->stream);
+      if (cr != 0) return cuda_fail(c, (cudaError_t)cr, "checked build: count kernel");
+#endif
       c->step += m;
       n_steps -= m;
     }
     if (n_steps == 0) return LBM_OK;
   }
+#ifndef LBM_CHECKED
   const int64_t G = c->graph_steps;
   if (G > 0 && n_steps >= G && !diag_last && !c->prof) {
     // whole blocks of G steps as graph replays on the private stream
@@ -739,7 +750,7 @@ int run_steps(lbm_ctx* c, int64_t n_steps, bool diag_last) {
     int rc = lbm::launch_step(c->storage, c->d, p, ss, c->prof ? ev : nullptr);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "step kernels");
 #ifdef LBM_CHECKED
-    rc = lbm::launch_check_counts(c->d, c->stream);
+    rc = lbm::launch_check_counts(c->d, 1, c->stream);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "checked build: count kernel");
 #endif
     ++c->step;

@@ -536,6 +536,18 @@ __device__ __forceinline__ bool chk_site(int64_t y, int64_t n, int* err) {
   return true;
 }
 
+// The same for the 18 links of a bulk site (a neighbour is used on odd steps only).
+template <bool ODD>
+__device__ __forceinline__ bool chk_links(int64_t x, const int32_t* dsc, int64_t n, int* err) {
+  bool ok = true;
+  if constexpr (kChecked) {
+    ok = chk_site(x, n, err);
+    if constexpr (ODD)
+      for (int o = 0; o < 18; ++o) ok = chk_site(x + dsc[o], n, err) && ok;
+  }
+  return ok;
+}
+
 // A copy of a base pointer the compiler cannot identify with the original:
 // stores through it form their addresses anew instead of keeping the 19 load
 // addresses live through the collision (38 registers on even steps).
@@ -2078,6 +2090,16 @@ __device__ __forceinline__ void ens_prefetch(const EnsembleLaunch& e, int64_t g,
   if (p) bulk_prefetch_l2(reinterpret_cast<const S*>(p) + (int64_t)lane * np, kTile * sizeof(S));
 }
 
+// Checked builds: site x of the tile at P, and its neighbours, within the member.
+template <class S, bool ODD>
+__device__ __forceinline__ bool ens_links(const MemberDev* m, const S* P, int64_t x,
+                                          const int32_t* dsc) {
+  if constexpr (kChecked)
+    return chk_links<ODD>(P - static_cast<const S*>(m->d.pop) + x, dsc, m->d.n, m->d.err);
+  else
+    return true;
+}
+
 template <class S, bool ODD, int W>
 __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::one)
     k_bulk_ens(const EnsembleLaunch e, const StepParams p) {
@@ -2097,6 +2119,7 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::one)
   C om;
   if constexpr (std::is_same<C, double>::value) om = m->omega;
   else om = __int_as_float(dsc[19]);
+  if (!ens_links<S, ODD>(m, P, lane, dsc)) return;
   bulk_update<S, ODD>(P, (int64_t)dsc[18], (int64_t)lane, dsc, om, m, nullptr);
 }
 
@@ -2129,9 +2152,14 @@ __global__ void __launch_bounds__(W * 32, EnsBulkMinBlocks<S, W>::two)
     const int32_t* dsc = lane < 16 ? da : db;
     S* P = ens_pop<S>(dsc);
     if (!P) return;  // padding
-    bulk_update2<S, ODD>(P, np, (int64_t)(2 * (lane & 15)), dsc, om, m, nullptr);
+    const int x = 2 * (lane & 15);
+    if (!ens_links<S, ODD>(m, P, x, dsc) || !ens_links<S, ODD>(m, P, x + 1, dsc)) return;
+    bulk_update2<S, ODD>(P, np, (int64_t)x, dsc, om, m, nullptr);
   } else {
     S* PA = ens_pop<S>(da);
+    if (kChecked && !__all_sync(0xFFFFFFFFu, ens_links<S, ODD>(m, PA, lane, da) &&
+                                                 (!PB || ens_links<S, ODD>(m, PB, lane, db))))
+      return;
     if (!PB) {
       bulk_update<S, ODD>(PA, np, (int64_t)lane, da, om, m, nullptr);
       return;
@@ -2481,8 +2509,13 @@ __global__ void __launch_bounds__(SmallCfg<S>::warps * 32, 1)
     } else if (k < d.n_tiles) {
       const int64_t x = (int64_t)dsc[19] * kTile + lane;
       const C om = omega_as<C>(p.omega, p.omega_f);
-      if (odd) bulk_update<S, true>(static_cast<S*>(d.pop), d.npad, x, dsc, om, d.err, d.chk);
-      else bulk_update<S, false>(static_cast<S*>(d.pop), d.npad, x, dsc, om, d.err, d.chk);
+      S* P = static_cast<S*>(d.pop);
+      if (odd) {
+        if (chk_links<true>(x, dsc, d.n, d.err))
+          bulk_update<S, true>(P, d.npad, x, dsc, om, d.err, d.chk);
+      } else if (chk_links<false>(x, dsc, d.n, d.err)) {
+        bulk_update<S, false>(P, d.npad, x, dsc, om, d.err, d.chk);
+      }
     }
     if (s + 1 < n_steps && !small_barrier(bar, base + (unsigned long long)(s + 1) * gridDim.x, d.err))
       return;
@@ -2697,12 +2730,13 @@ __device__ double block_sum(double v, double* sh) {
   return sh[0];
 }
 
-// Checked builds: every slot of a valid site stored exactly once since the
-// last check, padding slots never; the counts are cleared for the next step.
-__global__ void k_check_counts(int* chk, int64_t total, int64_t npad, int64_t n, int* err) {
+// Checked builds: every slot of a valid site stored exactly once a step since the
+// last check, padding slots never; the counts are cleared for the next one.
+__global__ void k_check_counts(int* chk, int64_t total, int64_t npad, int64_t n, int steps,
+                               int* err) {
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
        q += (int64_t)gridDim.x * blockDim.x) {
-    const int want = (q % npad) < n ? 1 : 0;
+    const int want = (q % npad) < n ? steps : 0;
     if (chk[q] != want) atomicOr(err, kErrCheck);
     chk[q] = 0;
   }
@@ -3185,11 +3219,11 @@ int launch_advance(int64_t* step_dev, int64_t by, void* stream) {
   return (int)cudaGetLastError();
 }
 
-int launch_check_counts(const DevLattice& d, void* stream) {
+int launch_check_counts(const DevLattice& d, int steps, void* stream) {
   if (!d.chk) return 0;
   const int64_t total = (int64_t)kQ * d.npad;
   k_check_counts<<<blocks_for(total, 256) < 4096 ? blocks_for(total, 256) : 4096, 256, 0,
-                   (cudaStream_t)stream>>>(d.chk, total, d.npad, d.n, d.err);
+                   (cudaStream_t)stream>>>(d.chk, total, d.npad, d.n, steps, d.err);
   return (int)cudaGetLastError();
 }
 

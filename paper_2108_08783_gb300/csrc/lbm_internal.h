@@ -394,7 +394,7 @@ int diag_blocks(int n_iolets, int fpi);
 int diag_flux_blocks(int64_t max_sites);
 // Checked builds: flag every population slot not stored exactly once since the
 // last call (padding slots: never), then clear the counts.
-int launch_check_counts(const DevLattice& d, void* stream);
+int launch_check_counts(const DevLattice& d, int steps, void* stream);  // since the last check
 
 // Learned warm start (mlp.cu): the network's forward pass on a given stream
 // (n rows in chunks of its batch size, using its activation buffers), its
