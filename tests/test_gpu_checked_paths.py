@@ -3,6 +3,11 @@ launched kernels: all steps of a small lattice in one launch, and ensembles, in
 every storage and pairing of the bulk kernels, with 4 and 8 warps per CTA and
 with graphs and members of odd and even numbers of bulk tiles.
 
+The same build takes the descending odd steps of populations beyond L2 on these
+small ones (-DLBM_ALTERNATE_BYTES=0): ensembles, and single lattices' launched
+kernels in pairings 1 to 4, with uniform and per-site walls, sites linked to two
+iolets, and diagnostic steps.
+
 Neighbour indices are range-checked in all of them (LBM_ECHECK from the next
 sync), the stores of the one launch are counted over its steps, and the fields
 are those of the package's build, bit for bit.
@@ -38,9 +43,36 @@ def _lat(geo, storage, k=0, wall="elastic"):
     return lat
 
 
+def _launched():
+    """Single lattices through the two launched kernels of a step."""
+    out = []
+    geos = [I.tube(7.5, 255, u_mean=0.02, u_amp=0.01, period=37.0), I.closed_box(3, 3, 35),
+            I.murray_tree(seed=3, depth=2, root_radius=7.0),
+            I.random_labels(4, (14, 11, 3), fill=0.8)]  # sites linked to two iolets
+    for storage in ("f32", "f16s", "bf16s"):
+        for mode in (1, 2, 3, 4):
+            for k, geo in enumerate(geos):
+                for warps in (4, 8):
+                    lat = _lat(geo, storage)
+                    if warps == 8 and lat.n_wall:  # F and kappa of every wall site
+                        w = np.arange(lat.n_wall)
+                        lat.set_wall("elastic", rho0=1.0, F=0.7 + 0.02 * (w % 7),
+                                     kappa=2.0 + w % 5)
+                    lat.tune(bulk_sites=mode, bulk_warps=warps, graph_steps=0,
+                             prefetch=(0, 3, 64, 4096)[k])
+                    diag = []
+                    for n in (1, 2, 2, 4):
+                        lat.step(n)
+                        diag.append(lat.step_diag(n))
+                    lat.sync()
+                    out += [lat.populations(), np.array(diag), *lat.wall_state()]
+                    lat.close()
+    return out
+
+
 def run():
     from paper_2108_08783_gb300 import Ensemble
-    out = []
+    out = _launched()
     geos = [I.tube(7.5, 150, u_mean=0.02, u_amp=0.01, period=37.0), I.closed_box(3, 3, 34),
             I.murray_tree(seed=3, depth=2, root_radius=7.0), I.random_labels(1, (17, 15, 21))]
     for storage in ("f64", "f32", "f16s", "bf16s"):
@@ -61,7 +93,8 @@ def run():
                 members = [_lat(g, storage, k) for k, g in enumerate(geos)]
                 assert [int(m.info()[4]) & 1 for m in members] == [1, 1, 0, 1]
                 ens = Ensemble(members)
-                ens.tune(bulk_sites=mode, bulk_warps=warps, graph_steps=2)
+                ens.tune(bulk_sites=mode, bulk_warps=warps, graph_steps=2,
+                         prefetch=5 if warps == 8 else 0)
                 for n in (1, 4, 3):
                     ens.step(n)
                     ens.sync()
@@ -72,7 +105,8 @@ def run():
 
 def test_checked_paths_are_clean_and_equal(tmp_path):
     from paper_2108_08783_gb300 import build
-    lib = build.build(out=str(tmp_path / "liblbm_checked.so"), extra=["-DLBM_CHECKED"])
+    lib = build.build(out=str(tmp_path / "liblbm_checked.so"),
+                      extra=["-DLBM_CHECKED", "-DLBM_ALTERNATE_BYTES=0"])
     res = str(tmp_path / "out.npz")
     r = subprocess.run([sys.executable, "-c", SCRIPT, ROOT, res],
                        env=dict(os.environ, LBM_LIBRARY=lib), capture_output=True, text=True,
