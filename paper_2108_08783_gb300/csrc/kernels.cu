@@ -1779,11 +1779,17 @@ __global__ void __launch_bounds__(kStageWarps * 32, kStages <= 2 ? 8 : (kStages 
     collide2<true, int*>(
         [&](int j) -> F2 { return Cd::unpack(row[j * (kTile / 2)]); },
         [&](int j) -> F2 { return Cd::unpack(lds_volatile_u32(row + j * (kTile / 2))); }, om,
-        d.err, [&](F2 s0) { Cd::st_al(P + x, s0); },
+        d.err,
+        [&](F2 s0) {
+          Cd::st_al(P + x, s0);
+          chk_count2(d.chk, P, P + x, kQ * np, d.err);
+        },
         [&](auto A, F2 sa, F2 sb) {
           constexpr int a = decltype(A)::value, b = a + 1;
           Cd::st_al(P + b * np + x, sa);
           Cd::st_al(P + a * np + x, sb);
+          chk_count2(d.chk, P, P + b * np + x, kQ * np, d.err);
+          chk_count2(d.chk, P, P + a * np + x, kQ * np, d.err);
         });
     __syncwarp();
     for (int i = 0; i < kStages; ++i) {

@@ -5,7 +5,7 @@ with graphs and members of odd and even numbers of bulk tiles.
 
 The same build takes the descending odd steps of populations beyond L2 on these
 small ones (-DLBM_ALTERNATE_BYTES=0): ensembles, and single lattices' launched
-kernels in pairings 1 to 4, with uniform and per-site walls, sites linked to two
+kernels in every pairing (staged rows too), with uniform and per-site walls, sites linked to two
 iolets, and diagnostic steps.
 
 Neighbour indices are range-checked in all of them (LBM_ECHECK from the next
@@ -50,7 +50,7 @@ def _launched():
             I.murray_tree(seed=3, depth=2, root_radius=7.0),
             I.random_labels(4, (14, 11, 3), fill=0.8)]  # sites linked to two iolets
     for storage in ("f32", "f16s", "bf16s"):
-        for mode in (1, 2, 3, 4):
+        for mode in (1, 2, 3, 4) if storage == "f32" else (1, 2, 3, 4, 5):
             for k, geo in enumerate(geos):
                 for warps in (4, 8):
                     lat = _lat(geo, storage)
