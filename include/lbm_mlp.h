@@ -45,9 +45,10 @@ typedef struct lbm_adam {
 } lbm_adam;
 
 /* lbm_mlp_create - a network with zero parameters.  max_batch >= 1 rows per
- * training step (forward passes of more rows run in chunks of max_batch);
- * the activation buffers (about 2 (n_in + 2 width (n_layers + 1)) bytes per
- * row) are allocated here.  alloc may be NULL (cudaMalloc); cuda_stream NULL
+ * training step.  A forward pass takes any number of rows: networks of 2 to 16
+ * layers up to 256 wide in one launch, others in chunks of max_batch.  What a
+ * training step keeps of its activations and errors (about 4 width n_layers
+ * bytes per row, at most) is allocated here.  alloc may be NULL (cudaMalloc); cuda_stream NULL
  * is the legacy default stream.  LBM_EINVAL for sizes outside the limits. */
 int lbm_mlp_create(int32_t n_in, int32_t width, int32_t n_layers, int32_t n_out,
                    int64_t max_batch, const lbm_allocator *alloc, void *cuda_stream,

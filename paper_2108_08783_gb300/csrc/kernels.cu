@@ -23,11 +23,16 @@
 //   velocity inlet: the GZS form with (rho, u_in(x, n));
 //   density outlet: the GZS form with (rho_out, u).
 //
-// One kernel per step (k_step), one warp per tile of 32 sites: bulk tiles
-// (all 18 links fluid) take a branch-free path with 18 neighbour offsets per
-// tile; boundary tiles first stage their per-site link data (link masks, F,
-// kappa, inlet profile and, on odd steps, per-site neighbours) into shared
-// memory with cp.async.bulk copies completing on an mbarrier.
+// A step is two kernels side by side, one warp per tile of 32 sites (or per two
+// bulk tiles): k_bulk / k_bulk2 for the tiles whose 18 links are all fluid, a
+// branch-free path with 18 neighbour offsets per tile, and k_boundary for the
+// others, which first load their per-site link data (link masks, inlet profile,
+// F and kappa where they differ between sites and, on odd steps of irregular
+// tiles, offsets by runs of lanes or per-site neighbours, the latter by
+// cp.async.bulk copies completing on an mbarrier).  Sites linked to two or more
+// iolets have a kernel of their own (k_boundary_multi), ensembles the same
+// kernels over all members' tiles (k_bulk_ens, k_bulk2_ens, k_boundary_ens).
+// Small lattices take all steps of a call in one launch, k_small.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda.h>
@@ -1124,11 +1129,12 @@ __device__ __forceinline__ typename Codec<S>::C boundary_fast(const D& d,
     }
   });
   const Mom<C> m = moments(g);
-  // FP32 compute: g stays in registers through the boundary rule (at 72
-  // registers no spills; parking it in shared memory and reading it back
-  // pair by pair, needed at 64, measured 1.5-3 % slower).  FP64: g is parked
-  // in the warp's area and read back pair by pair (volatile, so the 19
-  // doubles are not held in registers through the rule).
+  // FP32 compute: g stays in registers through the boundary rule (at 64
+  // registers odd steps spill 16 bytes a thread, 32 with the fused diagnostics,
+  // even steps none; parking g in shared memory and reading it back pair by
+  // pair measured 1.5-3 % slower).  FP64: g is parked in the warp's area and
+  // read back pair by pair (volatile, so the 19 doubles are not held in
+  // registers through the rule).
   constexpr bool kPark = std::is_same<C, double>::value;
   if constexpr (kPark) {
     unroll<kQ>([&](auto J) {
@@ -2449,8 +2455,8 @@ struct SmallCfg {
 // Grid barrier on a counter that only grows: every launch of a lattice adds a
 // multiple of its (fixed) grid to it, so the first value a CTA reads, before
 // its own first arrival and hence before anyone's second, gives the launch's
-// base; a launch replayed from a caller's graph needs nothing reset. One
-// release-add and an acquiring poll per CTA; bounded spin, false on timeout.
+// base, and nothing is reset between launches. One release-add and an acquiring
+// poll per CTA; bounded spin, false on timeout (lbm_sync then clears the counter).
 __device__ __forceinline__ bool small_barrier(unsigned long long* bar, unsigned long long target,
                                               int* err) {
   __syncthreads();
@@ -2478,7 +2484,7 @@ __global__ void __launch_bounds__(SmallCfg<S>::warps * 32, 1)
   using C = typename Codec<S>::C;
   using Cfg = SmallCfg<S>;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* mine = smem + w * Cfg::per_warp;
   int32_t* stage = reinterpret_cast<int32_t*>(mine);
   C* area = reinterpret_cast<C*>(mine + Cfg::stage);

@@ -180,9 +180,12 @@ __device__ __forceinline__ void stage_inputs(unsigned char* image, const float* 
 // through a ring of 16 KB stages (32 input features of the layer's rows each, one
 // bulk copy: 32 copies of 512 bytes a stage held the products back to half rate).
 // Warps 0-7 are the epilogue, warp 8 fills the ring, one lane of warp 9 issues
-// the MMAs.  The epilogue's tanhf bounds it (50 M of them for 65,536 rows of
-// the 4 x 256 network), so two CTAs share an SM (2 x 112 KB of shared memory,
-// 2 x 256 accumulator columns): one's products run under the other's
+// the MMAs.  Its epilogues bound it (50 M tanhf for 65,536 rows of the 4 x 256
+// network), by latency as much as by instructions: 56 % of the issue slots are
+// used at 30 % of the warps, 4.5 stalls an issue wait for a tensor-memory or
+// global load (each warp has one load of 8 columns in flight), and a tanh of half
+// the instructions gained nothing.  So two CTAs share an SM (2 x 112 KB of shared
+// memory, 2 x 256 accumulator columns): one's products run under the other's
 // epilogue.  nb is chosen so that the tiles fill whole rounds of 2 CTAs per SM.
 // 65,536 rows of the 4 x 256 network: 219 us layer by layer, 59 us so; the
 // pass of a warm start of 926,000 sites (227 chunks of 4,096 rows before, about
