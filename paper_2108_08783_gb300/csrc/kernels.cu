@@ -2559,6 +2559,11 @@ __global__ void k_set_step(int64_t* step, int64_t value) { *step = value; }
 // local array of neighbours in a rolled loop kept it (and the populations) in
 // local memory: k_moments took 312 us on the 5.1 M-site tube in FP16 and takes
 // 75 us so (362 MB, 0.7 of the measured HBM rate).
+// Odd layouts: all neighbours are loaded before the first index is handed out,
+// and the choice between the site's own slot and a neighbour's is a select. A
+// branch by direction with the neighbour's load inside made 18 dependent trips
+// to memory of it (k_moments on a tree of 4.3 M sites: FP32 203 us, 106 so;
+// FP16 174, 98; the rolled loop 111 and 252).
 template <class F>
 __device__ __forceinline__ void for_slots(const DevLattice& d, int64_t x, bool odd, F&& f) {
   f(std::integral_constant<int, 0>{}, x);
@@ -2570,23 +2575,25 @@ __device__ __forceinline__ void for_slots(const DevLattice& d, int64_t x, bool o
     return;
   }
   const TileDesc& td = d.tiles[x >> 5];
-  if (td.mask == 0) {
-    unroll<kQ - 1>([&](auto I) {
-      constexpr int j = decltype(I)::value + 1, o = dir_opp(j);
-      f(std::integral_constant<int, j>{}, o * d.npad + x + td.code[o - 1]);
-    });
-    return;
-  }
+  const uint32_t tmask = td.mask;
   const int64_t slot = (int64_t)td.slot + (x & 31);
-  const uint32_t nf = d.slot_mask[slot] & kDirBits;
-  const bool irr = td.mask & kIrregular;
+  const uint32_t nf = tmask ? d.slot_mask[slot] & kDirBits : 0u;
+  int32_t y[kQ - 1];
+  if (tmask & kIrregular)  // warp-uniform
+    unroll<kQ - 1>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      y[i] = d.slot_nbr[i * d.slot_stride + slot];
+    });
+  else
+    unroll<kQ - 1>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      y[i] = (int32_t)x + td.code[i];
+    });
   unroll<kQ - 1>([&](auto I) {
     constexpr int j = decltype(I)::value + 1, o = dir_opp(j);
-    int64_t q = j * d.npad + x;  // the site's own slot: the link opp(j) leaves the fluid
-    if (!((nf >> o) & 1u))
-      q = o * d.npad + (irr ? (int64_t)d.slot_nbr[(o - 1) * d.slot_stride + slot]
-                            : x + td.code[o - 1]);
-    f(std::integral_constant<int, j>{}, q);
+    // the site's own slot when the link opp(j) leaves the fluid
+    f(std::integral_constant<int, j>{},
+      (nf >> o) & 1u ? j * d.npad + x : o * d.npad + (int64_t)y[o - 1]);
   });
 }
 
