@@ -1679,8 +1679,12 @@ __device__ __forceinline__ float bulk_pair_warp(const BulkView& d, int64_t k0, f
 // at launch positions n_boundary + 2 (b W + w) and the one after it).
 // DIAG: also write the tiles' sums of rho - 1 (fused diagnostics), a separate
 // instantiation so that ordinary steps keep their registers.
+//
+// DIAG in 16-bit storage: 7 CTAs per SM (72 registers); at 64 the sums kept
+// through the stores made the odd kernel spill 130 bytes a thread (a diagnostic
+// step of the long tube, FP16: 120 us, 114 so).
 template <class S, bool ODD, bool VERT, int W, bool DIAG = false>
-__global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::two)
+__global__ void __launch_bounds__(W * 32, DIAG && sizeof(S) == 2 ? 7 : BulkMinBlocks<S, W>::two)
     k_bulk2(const DevLattice d, const StepParams p) {
   __shared__ __align__(16) int32_t desc_s[W][2][20];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1824,7 +1828,9 @@ __global__ void __launch_bounds__(W * 32, BulkMinBlocks<S, W>::one)
 
 // Resident CTAs (4 warps) per SM requested of the boundary kernel: 8, i.e. 64
 // registers, against 7 (72) and 6: depth-6 tree of root radius 36 FP32 138.5,
-// 139.8, 143.1 us a step, FP16 106.9, 108.7, 112.6; long tube within 0.1 %.
+// 139.8, 143.1 us a step, FP16 106.9, 108.7, 112.6; long tube within 0.1 %. With
+// the fused diagnostics 7: 8 spill (diagnostic step of a tree of root radius 30,
+// FP32: 124.9 us with 8, 122.2 with 7).
 #ifndef LBM_BOUNDARY_MINB
 #define LBM_BOUNDARY_MINB 8
 #endif
@@ -1998,7 +2004,8 @@ __device__ __forceinline__ bool boundary_tile(const D& d, const StepParams& p, i
 }
 
 template <class S, bool ODD, bool DIAG = false>
-__global__ void __launch_bounds__(kBoundaryWarps * 32, sizeof(S) == 8 ? 2 : LBM_BOUNDARY_MINB)
+__global__ void __launch_bounds__(kBoundaryWarps * 32,
+                                  sizeof(S) == 8 ? 2 : (DIAG ? 7 : LBM_BOUNDARY_MINB))
     k_boundary(const DevLattice d, const StepParams p0) {
   StepParams p = p0;
   p.diag = DIAG;  // a compile-time constant for the tile code
@@ -2321,9 +2328,9 @@ __device__ bool grid_sync(GridSync* gs, unsigned expected, unsigned& gen, int ne
 // The four tile bodies as separate functions, so that each keeps the
 // register allocation it has in its own kernel. Each forms its step's parameters
 // itself from the member's table: a copy per tile in local memory, handed over by
-// reference, cost 4 to 8 % of a step (24 tubes: FP16 52.4 us, 50.0 so; FP32 55.6, 52.2), and what an
-// ensemble never sets (fused diagnostics, descending order, one F and kappa) is
-// known here when the bodies are compiled.
+// reference, cost 4 to 8 % of a step (24 tubes: FP16 52.4 us, 50.0 so; FP32 55.6,
+// 52.2), and what an ensemble never sets (fused diagnostics, descending order, one
+// F and kappa) is known here when the bodies are compiled.
 __device__ __forceinline__ StepParams member_params(const MemberDev& md, int64_t step) {
   StepParams p{};
   p.omega = md.omega;
