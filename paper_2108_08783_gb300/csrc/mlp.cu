@@ -861,12 +861,11 @@ int lbm_mlp_set_params(lbm_mlp* net, const float* theta, int32_t src_is_device) 
   if (!e) e = (int)cudaMemsetAsync(net->m, 0, bytes, s);
   if (!e) e = (int)cudaMemsetAsync(net->v, 0, bytes, s);
   if (!e) {
-    k_to_bf16<<<grid_for(net->n_params, 256), 256, 0, s>>>(net->theta, net->w16, net->n_params);
-    e = (int)cudaGetLastError();
-  }
-  if (!e && net->fused) {
-    k_pack<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(net->w16, net->pmap, net->wpack,
-                                                                  net->n_params);
+    if (net->fused)
+      k_round_pack<<<(unsigned)ceil_div(net->n_params, 256), 256, 0, s>>>(
+          net->theta, net->w16, net->pmap, net->wpack, net->n_params);
+    else
+      k_to_bf16<<<grid_for(net->n_params, 256), 256, 0, s>>>(net->theta, net->w16, net->n_params);
     e = (int)cudaGetLastError();
   }
   if (!e) e = (int)cudaStreamSynchronize(s);
